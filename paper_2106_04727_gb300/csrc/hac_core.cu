@@ -1817,6 +1817,57 @@ struct RoundTimes {
   bool trace = false;
 };
 
+// Whether rounds over K active clusters may run in one launch (hac_finish.cu).
+// Below the capacity one launch beats the ordinary rounds at every size
+// measured (whole runs from the points, Ward, ms, one launch / rounds: 2-D
+// 64 points 0.17 / 1.75, 1,024 0.38 / 3.15, 4,096 0.87 / 4.01; 16-D 64 points
+// 0.42 / 2.42, 2,048 1.37 / 5.37), so the line is the capacity itself.
+bool finish_ok(const hac_ctx *h, int64_t K) {
+  const State &s = h->s;
+  return closed_form(s.linkage) && s.max_inst == 1 && !s.noprune && K > 1 && K <= fin_cap(s.d);
+}
+
+// One launch of at most `limit` rounds (0 = to the end) from the current
+// lists, or from the input points (direct, with the dendrogram written to
+// `out`); the counters of the launch come back in *c.
+int run_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64_t limit,
+               bool direct, hac_merge *out, int32_t *out_round, Counters *c) {
+  State &s = h->s;
+  FinArgs a{};
+  a.s = s;
+  a.K = K;
+  a.nterm = nterm;
+  a.round = round;
+  a.rounds_max = (int)std::min<int64_t>(limit, INT32_MAX / 2);
+  a.scale = s.coord_scale;
+  a.order = s.order[h->ocur];
+  a.order_out = s.order[h->ocur];
+  if (direct) {
+    a.raw = h->raw;
+    a.in_f32 = h->dt == HAC_F32;
+    a.out = out;
+    a.out_round = out_round;
+    a.n_rec = K - 1;
+    CK(cudaMemsetAsync(s.ctr, 0, sizeof(Counters), st));
+  }
+  int rc = launch_finish(a, st);
+  if (rc) return rc;
+  h->launches += 1;
+  CK(cudaMemcpyAsync(c, s.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  return HAC_OK;
+}
+
+// rounds per launch: all of them, or few where a time limit is checked
+int64_t finish_limit(const hac_opts &opt, int round) {
+  int64_t lim = opt.timeout_s > 0 ? 8 : 0;
+  if (opt.max_rounds) {
+    const int64_t left = opt.max_rounds - round;
+    lim = lim ? std::min(lim, left) : left;
+  }
+  return lim;
+}
+
 // Algorithm 1's rounds from the initial layout until one cluster is left:
 // round_step, tree rebuild, then the round's counters are read and checked.
 // HAC_ETIMEOUT once a limit of `opt` is reached (checked between rounds).
@@ -1834,6 +1885,31 @@ int run_rounds(hac_ctx *h, const hac_opts &opt, cudaStream_t st, RoundCtl &ctl, 
         std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count() >
             opt.timeout_s)
       return HAC_ETIMEOUT;
+    if (finish_ok(h, K) && s.coord_scale >= (float)FIN_SCALE_LO &&
+        s.coord_scale < (float)FIN_SCALE_HI) {
+      if (tm) cudaEventRecord(tm->e0, st);
+      rc = run_finish(h, st, K, nterm, round, finish_limit(opt, round), false, nullptr, nullptr,
+                      &c);
+      if (rc) return rc;
+      if ((c.err & ~ERR_NONFINITE) || c.nactive >= K) return HAC_EINTERNAL;
+      if (tm) {
+        cudaEventRecord(tm->e3, st);
+        CK(cudaEventSynchronize(tm->e3));
+        float ms;
+        cudaEventElapsedTime(&ms, tm->e0, tm->e3);
+        tm->ms_nn += ms;
+        if (trace)
+          fprintf(stderr, "hac rounds %d .. %d in one launch: K %d -> %d, %.3f ms\n", round,
+                  round + c.fin_rounds - 1, K, c.nactive, ms);
+      }
+      K = c.nactive;
+      nterm = c.nterm;
+      round += c.fin_rounds;
+      ctl.searches += c.fin_searches;
+      ctl.naive += c.fin_naive;
+      *rounds_out = round;
+      continue;
+    }
     if (tm) cudaEventRecord(tm->e0, st);
     const int big_iters0 = ctl.big_iters, big_reqs0 = ctl.big_reqs;
     ctl.naive += (int64_t)nterm * (K - 1);
@@ -1888,6 +1964,40 @@ int run_rounds(hac_ctx *h, const hac_opts &opt, cudaStream_t st, RoundCtl &ctl, 
     ++round;
     *rounds_out = round;
   }
+  return HAC_OK;
+}
+
+// Algorithmic bytes of the searches (true dimension d, not padded):
+// node test = centroid box (+ complete's hi-min / lo-max) + min size;
+// leaf slot = order entry + FP32 centroid + size (+ complete's box);
+// evaluated pair = Ward FP64 centroid, or the point rows of both clusters;
+// per terminal = its own centroid, box, size and pred word.
+int64_t query_bytes(const hac_ctx *h, const Counters &c, int64_t searches) {
+  const int64_t d = h->d;
+  const int64_t ew = 8;  // FP64 path
+  const bool comp = h->s.linkage == LK_COMPLETE;
+  const int64_t node_b = 2 * d * 4 + 4 + (comp ? 2 * d * 4 : 0);
+  const int64_t leaf_b = 4 + d * 4 + 4 + (comp ? 2 * d * 4 : 0);
+  const int64_t term_b = d * 4 + 2 * d * 4 + 4 + 8 + 4 + 16;
+  return (int64_t)c.nodes * node_b + (int64_t)c.ltests * leaf_b + searches * term_b +
+         (int64_t)(closed_form(h->s.linkage) ? c.cluster_pairs : c.prows) * d * ew;
+}
+
+// A whole run in one launch, where the instance and the options allow it:
+// the dendrogram goes to out / out_round.  *done = 0 if the ordinary path has
+// to run instead.
+int run_direct(hac_ctx *h, const hac_opts &opt, cudaStream_t st, hac_merge *out,
+               int32_t *out_round, Counters *c, int *done) {
+  *done = 0;
+  if (!finish_ok(h, h->n) || opt.max_rounds || opt.timeout_s > 0) return HAC_OK;
+  const int n = (int)h->n;
+  h->ocur = h->pcur = 0;
+  int rc = run_finish(h, st, n, n, 0, 0, true, out, out_round, c);
+  if (rc) return rc;
+  if (c->err & ERR_NONFINITE) return HAC_EINVAL;
+  if (c->fin_refused) return HAC_OK;
+  if (c->err || c->nmerges != n - 1) return HAC_EINTERNAL;
+  *done = 1;
   return HAC_OK;
 }
 
@@ -1951,11 +2061,34 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
   h->st = hac_stats_t{};
   h->st.device_bytes = h->bytes;
   const auto t0 = std::chrono::steady_clock::now();
+  auto ms_since_t0 = [&] {
+    return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+  };
+  h->launches = 0;
+  {
+    Counters c{};
+    int direct = 0;
+    const int rc = run_direct(h, opt, st, h->dout, h->dout_round, &c, &direct);
+    if (rc) return rc;
+    if (direct) {
+      hac_stats_t &r = h->st;
+      h->n_merges = r.merges = c.nmerges;
+      r.rounds = c.fin_rounds;
+      r.nn_searches = c.fin_searches;
+      r.naive_pairs = c.fin_naive;
+      r.cluster_pairs = (int64_t)c.cluster_pairs;
+      r.leaf_tests = (int64_t)c.ltests;
+      r.query_bytes = query_bytes(h, c, r.nn_searches);
+      r.kernel_launches = h->launches;
+      r.ms_nn = r.ms_total = ms_since_t0();  // one launch: not split into phases
+      h->done = true;
+      return HAC_OK;
+    }
+  }
   Ev e0, e1, e2, e3, eq0, eq1, eb0, eb1;
   double ms_nn = 0, ms_merge = 0, ms_update = 0, ms_init = 0, ms_query = 0, ms_big = 0;
   int64_t big_launch = 0;
   int64_t qlaunch = 0;
-  h->launches = 0;
   cudaEventRecord(e0.e, st);
   int rc = h->dt == HAC_F32 ? init_layout<float>(h, st) : init_layout<double>(h, st);
   if (rc) return rc;
@@ -2024,31 +2157,11 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
   h->st.dense_rechecks = ctl.dense_rechecks;
   h->st.ms_dense = ctl.ms_dense;
   h->st.point_pairs += (int64_t)(c.dense_pp + c.dense_rq_pp);
-  {
-    // algorithmic bytes of the search kernel (true dimension d, not padded):
-    // node test = centroid box (+ complete's hi-min / lo-max) + min size;
-    // leaf slot = order entry + FP32 centroid + size (+ complete's box);
-    // evaluated pair = Ward FP64 centroid, or the point rows of both clusters;
-    // per terminal = its own centroid, box, size and pred word.
-    const int64_t d = h->d;
-    const int64_t ew = 8;  // FP64 path
-    const bool comp = s.linkage == LK_COMPLETE;
-    const int64_t node_b = 2 * d * 4 + 4 + (comp ? 2 * d * 4 : 0);
-    const int64_t leaf_b = 4 + d * 4 + 4 + (comp ? 2 * d * 4 : 0);
-    const int64_t term_b = d * 4 + 2 * d * 4 + 4 + 8 + 4 + 16;
-    int64_t qb = (int64_t)c.nodes * node_b + (int64_t)c.ltests * leaf_b +
-                 h->st.nn_searches * term_b;
-    if (closed_form(s.linkage))
-      qb += (int64_t)c.cluster_pairs * d * ew;
-    else
-      qb += (int64_t)c.prows * d * ew;
-    h->st.query_bytes = qb;
-  }
+  h->st.query_bytes = query_bytes(h, c, h->st.nn_searches);
   h->st.ms_nn = ms_nn;
   h->st.ms_merge = ms_merge;
   h->st.ms_update = ms_update;
-  h->st.ms_total =
-      std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+  h->st.ms_total = ms_since_t0();
   h->done = true;
   return HAC_OK;
 }
@@ -2284,14 +2397,17 @@ bool carve_state(hac_ctx &h, Carver &cv) {
 int static_run(hac_ctx &h, const hac_opts &opt, cudaStream_t st, hac_merge *dev_out) {
   State &s = h.s;
   const auto t0 = std::chrono::steady_clock::now();
-  int rc = h.dt == HAC_F32 ? init_layout<float>(&h, st) : init_layout<double>(&h, st);
+  Counters c{};
+  int direct = 0;
+  int rc = run_direct(&h, opt, st, dev_out, h.dout_round, &c, &direct);
+  if (rc || direct) return rc;
+  rc = h.dt == HAC_F32 ? init_layout<float>(&h, st) : init_layout<double>(&h, st);
   if (rc) return rc;
   if (s.p32_max >= FP32_COORD_LIMIT) s.prec = HAC_PREC_F64;  // FP32 would overflow
   RoundCtl ctl;  // no events: nothing is created here
   int rounds = 0;
   rc = run_rounds(&h, opt, st, ctl, nullptr, t0, &rounds);
   if (rc) return rc;
-  Counters c{};
   CK(cudaMemcpyAsync(&c, s.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (c.nmerges != h.n - 1) return HAC_EINTERNAL;

@@ -234,6 +234,24 @@ struct RoundCtl {
   int64_t dense_rechecks = 0;  // matrix entries re-scored in FP64
 };
 
+// Rounds of a closed-form linkage run in one launch (hac_finish.cu): from the
+// active and terminal lists, or (raw set) from the input points
+struct FinArgs {
+  State s;
+  int K, nterm, round;   // active clusters, terminals, first round
+  int rounds_max;        // rounds to run at most (0 = to the end)
+  int Kc;                // staged capacity (set by the launch)
+  float scale;           // largest |coordinate| after recentring (not direct)
+  const int32_t *order;  // active cids
+  int32_t *order_out;    // where they go if the round limit stops the run
+  const void *raw;       // direct: the input points
+  int in_f32;            // their type
+  hac_merge *out;        // direct: the dendrogram in canonical order, and
+  int32_t *out_round;    //   each merge's round
+  int n_rec;             // direct: records to write
+};
+int launch_finish(FinArgs &a, cudaStream_t st);
+
 int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCtl &ctl,
                int *npairs_out);
 

@@ -33,6 +33,10 @@ struct Counters {
   unsigned long long big_skip;  // of those, pairs complete linkage skipped by box bounds
   int32_t nrq;       // dense phase: pairs listed for an FP64 re-score this pass
   unsigned long long dense_pp, dense_rq_pp;  // dense phase: sweep / re-score point pairs
+  // one-launch rounds (hac_finish.cu): rounds run, their searches and naive
+  // pairs; refused: the input's scale is not for that path
+  int32_t fin_rounds, fin_refused;
+  long long fin_searches, fin_naive;
 };
 
 enum : int32_t { ERR_NONFINITE = 1, ERR_NO_NN = 2, ERR_STACK = 4, ERR_WINDOW = 8, ERR_TREE = 16 };
@@ -303,6 +307,27 @@ __host__ __device__ inline int tree_caps(int K, int *cap) {
 // differences then stay below 2^86 even for d = 16 and Ward's weights.  Runs
 // over larger coordinates take the FP64 path in either precision mode.
 constexpr double FP32_COORD_LIMIT = 1099511627776.0;  // 2^40
+
+// One-launch rounds of the closed-form linkages (hac_finish.cu): at most
+// FIN_MAX_K active clusters, their staged records within FIN_SMEM bytes per
+// block, and a largest recentred coordinate in [FIN_SCALE_LO, FIN_SCALE_HI)
+// (from 2^-30 on the flush of squared distances below 2^-126 is far below
+// the error term of the FP32 centroids).
+constexpr int FIN_MAX_K = 4096;
+constexpr int FIN_SMEM = 200 * 1024;
+constexpr double FIN_SCALE_LO = 9.313225746154785e-10;  // 2^-30
+constexpr double FIN_SCALE_HI = 1099511627776.0;        // 2^40
+
+// dimension a record is staged with (zero-padded to it), and its bytes: the
+// coordinates, 1/size or variance, cid and terminal entry
+__host__ __device__ inline int fin_dim(int d) {
+  return d <= 6 ? d : d <= 8 ? 8 : d <= 10 ? 10 : d <= 12 ? 12 : 16;
+}
+__host__ __device__ inline int fin_record_bytes(int fd) { return 4 * fd + 12; }
+__host__ __device__ inline int fin_cap(int d) {
+  const int c = FIN_SMEM / fin_record_bytes(fin_dim(d)) & ~31;
+  return c < FIN_MAX_K ? c : FIN_MAX_K;
+}
 
 // tinfo entries after the per-level node counts
 constexpr int TI_TOP = MAXLEV + 1;    // lowest level with at most 32 nodes (the root's children)
