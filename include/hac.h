@@ -130,14 +130,14 @@ typedef struct {
   int64_t naive_pairs;       /* cluster pairs a search without range queries would
                                 evaluate: terminals x (active clusters - 1), summed
                                 over rounds */
-  int64_t dense_k;           /* average linkage: clusters active when the run switched
+  int64_t dense_k;           /* average, complete: clusters active when the run switched
                                 to the dense matrix of all their pair distances (0 = it
                                 did not) */
   int64_t dense_rounds;      /* rounds run on that matrix */
   int64_t dense_point_pairs; /* point pairs of the all-pairs sweep that filled it (also
                                 in point_pairs) */
   int64_t dense_rechecks;    /* FP32 mode: matrix entries re-scored in FP64 */
-  double ms_dense;           /* device time of the sweep */
+  double ms_dense;           /* device time of filling the matrix */
 } hac_stats_t;
 
 /* Default options (FP64, no cache, no limits, own stream).  No counterpart in
@@ -168,9 +168,14 @@ int hac_create_device(const void *dev_points, int64_t n, int d, hac_dtype dt, ha
  * clusters are active, to the full matrix of their pair distances (the
  * Section 5 cache with room for every pair: 24 bytes per entry of the K x K
  * matrix, allocated once per handle; without room for it the run stays on
- * the range-query search).  K is 8,192 for d <= 3, 16,384 for d <= 8 and
- * 65,536 above, capped so that the matrix takes at most half of the device
- * memory free when the run starts; the environment variable HAC_DENSE_K,
+ * the range-query search).  K is 4,096 to 8,192 for d <= 3 and 4,096 to 16,384
+ * for d <= 8, by n, and 65,536 above, capped so that the matrix takes at most
+ * half of the device memory free when the run starts.  Complete linkage runs
+ * on such a matrix (16 bytes per entry) from the first round on if it has at
+ * most K points: 24,576 to 32,768 by d and precision, capped the same way.  A
+ * run that starts on the matrix takes no cache.  Ward and avg-2 runs of at most
+ * 4,096 points (d <= 10; 2,688 in 16-D) take no matrix and no tree either: all
+ * their rounds are one launch.  The environment variable HAC_DENSE_K,
  * read at hac_create, sets it instead (0 = never).  opts may be NULL (defaults).  Blocks until done.  May be called
  * again on the same handle: each call recomputes from the stored points.
  * HAC_ETIMEOUT if a limit in opts is hit (the handle stays usable). */
@@ -214,7 +219,7 @@ const char *hac_strerror(int code);
  * synchronisation that cudaMalloc/cudaFree can cause).
  *
  * Same dendrogram as hac_create + hac_run + hac_dendrogram on the same points
- * and options (with the dense matrix of average linkage off, HAC_DENSE_K=0;
+ * and options (with the dense matrix off, HAC_DENSE_K=0;
  * with it on, the same tree and heights within the precision mode's stated
  * bound), computed by the same kernels, but all working memory comes
  * from a fixed 6 MiB device array inside the library, which every GPU that

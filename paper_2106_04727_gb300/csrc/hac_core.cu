@@ -1063,17 +1063,19 @@ __global__ void k_cmp_write(State s, const int32_t *order, int32_t *order_out, i
     order_out[ok] = c;
     s.pos[c] = ok;
     if (seg_out) seg_out[c] = os;
-    const int dp = s.dp;
-    for (int k = 0; k < dp; ++k) {
-      s.q32[(size_t)ok * dp + k] = s.cent32[(size_t)c * dp + k];
-      s.q64[(size_t)ok * dp + k] = s.cent[(size_t)c * dp + k];
-      s.qblo[(size_t)ok * dp + k] = s.blo[(size_t)c * dp + k];
-      s.qbhi[(size_t)ok * dp + k] = s.bhi[(size_t)c * dp + k];
+    if (!s.dense) {  // records of the range-query search
+      const int dp = s.dp;
+      for (int k = 0; k < dp; ++k) {
+        s.q32[(size_t)ok * dp + k] = s.cent32[(size_t)c * dp + k];
+        s.q64[(size_t)ok * dp + k] = s.cent[(size_t)c * dp + k];
+        s.qblo[(size_t)ok * dp + k] = s.blo[(size_t)c * dp + k];
+        s.qbhi[(size_t)ok * dp + k] = s.bhi[(size_t)c * dp + k];
+      }
+      s.qsz[ok] = sz;
+      s.qseg[ok] = os;
+      s.qvar[ok] = sz > 1 ? cluster_var_up(s, c, sz) : 0.f;
+      s.qinst[ok] = s.iseq[s.inst[c]];
     }
-    s.qsz[ok] = sz;
-    s.qseg[ok] = os;
-    s.qvar[ok] = sz > 1 ? cluster_var_up(s, c, sz) : 0.f;
-    s.qinst[ok] = s.iseq[s.inst[c]];
     if (ist) {
       s.term[ot] = c;
       s.isterm[c] = round + 1;
@@ -1089,9 +1091,10 @@ __global__ void k_relayout(State s, int pc, int64_t n) {  // n: points in the cu
     const int c = s.plab[pc][p];
     int r = c;
     int off = (int)p - s.seg[pc][c];
-    if (!s.alive[c]) {
-      r = s.rootof[c];
-      off += s.reloff[c];
+    // retired since the layout: the survivor has a smaller cid each time
+    while (!s.alive[r]) {
+      off += s.reloff[r];
+      r = s.rootof[r];
     }
     if (s.idone[s.inst[r]]) continue;  // finished instance: its points leave
     const int64_t q = (int64_t)s.seg[nx][r] + off;
@@ -1410,13 +1413,15 @@ int init_layout(hac_ctx *h, cudaStream_t st) {
   s.cur = 0;
   s.dense = 0;
   s.dk = 0;
+  h->lay_stale = 0;
   k_layout<T><<<grid_for(n, TPB), TPB, 0, st>>>(s, X, h->vals[sc], h->keys[sc], ctrp);
   CK(cudaGetLastError());
   Counters c{};
   c.nterm = (int)n;
   c.nactive = (int)n;
   CK(cudaMemcpyAsync(s.ctr, &c, sizeof(Counters), cudaMemcpyHostToDevice, st));
-  return build_tree(h, s.order[0], (int)n, st);
+  // (a run that starts on the dense matrix never searches the tree)
+  return h->dense_first ? HAC_OK : build_tree(h, s.order[0], (int)n, st);
 }
 
 // Canonical order of the merge records on the device, (height, size, cid_a)
@@ -1757,10 +1762,7 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
   if (npairs <= 0) return HAC_EINTERNAL;
   k_merge<<<grid_for(npairs, TPB), TPB, 0, st>>>(s, round, npairs);
   h->launches += 4;  // merge, 3 compaction kernels
-  if (dense) {
-    rc = dense_update(h, st, round, K, npairs);
-    if (rc) return rc;
-  } else if (s.cache_slots > 0) {
+  if (!dense && s.cache_slots > 0) {
     const int S = s.cache_slots;
     const size_t smem = (size_t)CM_WARPS * 5 * S * sizeof(CEntry);
     const int blocks = std::max(1, std::min(cdiv(npairs, CM_WARPS), device_sms() * 32));
@@ -1787,11 +1789,26 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
                                   round);
   CK(cudaGetLastError());
   h->ocur ^= 1;
+  if (dense) {
+    h->lay_stale = 1;
+    return dense_update(h, st, round, K, K - npairs);
+  }
   if (need_points) {
     k_relayout<<<grid_for(h->lay_n, TPB), TPB, 0, st>>>(s, h->pcur, h->lay_n);
     h->launches += 1;
     h->pcur ^= 1;
   }
+  return HAC_OK;
+}
+
+// The compaction has kept the clusters' segment starts in the spare seg array.
+int relayout_if_stale(hac_ctx *h, cudaStream_t st) {
+  if (!h->lay_stale) return HAC_OK;
+  k_relayout<<<grid_for(h->lay_n, TPB), TPB, 0, st>>>(h->s, h->pcur, h->lay_n);
+  CK(cudaGetLastError());
+  h->launches += 1;
+  h->pcur ^= 1;
+  h->lay_stale = 0;
   return HAC_OK;
 }
 
@@ -1878,6 +1895,7 @@ int run_rounds(hac_ctx *h, const hac_opts &opt, cudaStream_t st, RoundCtl &ctl, 
   int K = (int)h->n, nterm = (int)h->n, round = 0, rc = 0;
   Counters c{}, cprev{};
   const bool trace = tm && tm->trace;
+  int dfin_skip = 0, dfin_wait = 1;  // ordinary rounds before the next dense_finish
   *rounds_out = 0;
   while (K > 1) {
     if (opt.max_rounds && round >= opt.max_rounds) return HAC_ETIMEOUT;
@@ -1909,6 +1927,38 @@ int run_rounds(hac_ctx *h, const hac_opts &opt, cudaStream_t st, RoundCtl &ctl, 
       ctl.naive += c.fin_naive;
       *rounds_out = round;
       continue;
+    }
+    if (s.max_inst == 1 && !closed_form(s.linkage)) {
+      const int dense = dense_maybe_enter(h, st, K, ctl);
+      if (dense < 0) return dense;
+    }
+    if (s.dense && K <= DFIN_K && dfin_skip-- <= 0) {
+      if (tm) cudaEventRecord(tm->e0, st);
+      rc = dense_finish(h, st, K, nterm, round, finish_limit(opt, round), &c);
+      if (rc) return rc;
+      if (c.err & ~ERR_NONFINITE) return HAC_EINTERNAL;
+      if (tm) {
+        cudaEventRecord(tm->e3, st);
+        CK(cudaEventSynchronize(tm->e3));
+        float ms;
+        cudaEventElapsedTime(&ms, tm->e0, tm->e3);
+        tm->ms_nn += ms;
+        if (trace)
+          fprintf(stderr, "hac rounds %d .. %d in one launch: K %d -> %d, %.3f ms\n", round,
+                  round + c.fin_rounds - 1, K, c.nactive, ms);
+      }
+      // a re-score is due in this round (or came at once: the next ones may
+      // need it too, so ordinary rounds run for a while)
+      dfin_wait = c.fin_rounds ? 1 : std::min(2 * dfin_wait, 16);
+      dfin_skip = dfin_wait;
+      K = c.nactive;
+      nterm = c.nterm;
+      round += c.fin_rounds;
+      ctl.searches += c.fin_searches;
+      ctl.naive += c.fin_naive;
+      ctl.dense_rounds += c.fin_rounds;
+      *rounds_out = round;
+      if (c.fin_rounds) continue;
     }
     if (tm) cudaEventRecord(tm->e0, st);
     const int big_iters0 = ctl.big_iters, big_reqs0 = ctl.big_reqs;
@@ -2013,7 +2063,11 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
   s.noprune = (opt.flags & HAC_FLAG_NO_PRUNE) ? 1 : 0;
   h->done = false;
   // Section 5 cache tables (complete / average only: Ward distances are O(1))
-  const int slots = closed_form(s.linkage) ? 0 : std::min(opt.cache_slots, CACHE_MAX_SLOTS);
+  int slots = closed_form(s.linkage) ? 0 : std::min(opt.cache_slots, CACHE_MAX_SLOTS);
+  if (h->dense_k < 0 && !closed_form(s.linkage))
+    h->dense_def = std::max(dense_default(h->n, s.d, s.linkage, s.prec), h->dense_cap);
+  h->dense_first = dense_reserve(h, (int)h->n);
+  if (h->dense_first) slots = 0;  // every round runs on the matrix
   if (slots > h->cache_alloc_slots) {
     int rc0 = 0;
     // a larger table replaces the old one (a smaller request reuses it)
@@ -2093,7 +2147,6 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
   int rc = h->dt == HAC_F32 ? init_layout<float>(h, st) : init_layout<double>(h, st);
   if (rc) return rc;
   if (s.p32_max >= FP32_COORD_LIMIT) s.prec = HAC_PREC_F64;  // FP32 would overflow
-  if (h->dense_k < 0 && s.linkage == LK_AVERAGE) h->dense_def = dense_default(s.d);
   cudaEventRecord(e1.e, st);
   CK(cudaEventSynchronize(e1.e));
   {
@@ -2151,7 +2204,7 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
   h->st.big_point_pairs = (int64_t)(c.big_pp - c.big_skip);
   h->st.big_launches = big_launch;
   h->st.cache_lw_entries = (int64_t)c.cache_lw;
-  h->st.dense_k = s.dense ? s.dk : 0;
+  h->st.dense_k = s.dense ? h->dense_k0 : 0;
   h->st.dense_rounds = ctl.dense_rounds;
   h->st.dense_point_pairs = (int64_t)c.dense_pp;
   h->st.dense_rechecks = ctl.dense_rechecks;

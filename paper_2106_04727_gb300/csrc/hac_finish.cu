@@ -537,31 +537,10 @@ int launch_d(FinArgs &a, cudaStream_t st) {
     while (P < (size_t)a.n_rec) P <<= 1;
     smem = std::max(smem, P * 20);
   }
-  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.blockDim = dim3(FT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
   // blocks: a search is K / 32 steps of one warp, so few clusters need few
-  // blocks (a barrier of one block is cheaper than the cluster's); 16 where
-  // the device can place them, else the portable 8
-  int nct = a.K <= 96 ? 1 : a.K <= 320 ? 4 : a.K <= 640 ? 8 : 16;
-  for (;; nct >>= 1) {
-    cfg.gridDim = dim3(nct);
-    at.val.clusterDim.x = nct;
-    if (nct <= 8) break;
-    int can = 0;
-    if (cudaOccupancyMaxActiveClusters(&can, kern, &cfg) == cudaSuccess && can >= 1) break;
-    cudaGetLastError();
-  }
-  CK(cudaLaunchKernelEx(&cfg, kern, a));
-  return HAC_OK;
+  // blocks (a barrier of one block is cheaper than the cluster's)
+  const int nct = a.K <= 96 ? 1 : a.K <= 320 ? 4 : a.K <= 640 ? 8 : 16;
+  return launch_cluster((const void *)kern, nct, FT, smem, &a, st);
 }
 
 template <int LK>
@@ -581,6 +560,33 @@ int launch_lk_fin(FinArgs &a, cudaStream_t st) {
 }
 
 }  // namespace
+
+int launch_cluster(const void *kern, int nct, int threads, size_t smem, void *args,
+                   cudaStream_t st) {
+  if (smem > 48 * 1024)
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  if (nct > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  for (;; nct >>= 1) {  // 16 blocks where the device can place them, else the portable 8
+    cfg.gridDim = dim3(nct);
+    at.val.clusterDim.x = nct;
+    if (nct <= 8) break;
+    int can = 0;
+    if (cudaOccupancyMaxActiveClusters(&can, kern, &cfg) == cudaSuccess && can >= 1) break;
+    cudaGetLastError();
+  }
+  void *pa[1] = {args};
+  CK(cudaLaunchKernelExC(&cfg, kern, pa));
+  return HAC_OK;
+}
 
 int launch_finish(FinArgs &a, cudaStream_t st) {
   return a.s.linkage == LK_WARD ? launch_lk_fin<LK_WARD>(a, st) : launch_lk_fin<LK_AVG2>(a, st);

@@ -147,6 +147,13 @@ struct hac_ctx {
   int64_t dense_k = -1;  // -1: the default for the instance
   int64_t dense_def = 0;  // that default for the current run (dense_default)
   int64_t dense_cap = 0; // matrix dimension the buffers were allocated for
+  double *dense_buf = nullptr;  // the matrix buffers, dense_stride doubles each
+  size_t dense_stride = 0;
+  int dense_first = 0;   // the current run starts on the matrix
+  int64_t dense_k0 = 0;  // active clusters when the run switched to the matrix
+  // the point layout is older than the clusters: on the matrix points only
+  // move when a re-score needs them (relayout_if_stale)
+  int lay_stale = 0;
   int64_t launches = 0;  // kernels launched in the current run
   int ocur = 0, pcur = 0;
   bool done = false;
@@ -264,14 +271,26 @@ int big_finish(const State &s, int r0, int m, cudaStream_t st);
 int launch_big_complete(const State &s, int r0, cudaStream_t st);
 int launch_big_average(const State &s, int r0, cudaStream_t st);
 
-// dense phase (hac_dense.cu): whether this round should run on the matrix
-// (entering it if needed: allocation, the all-pairs sweep); the
-// nearest-neighbour search of the round's terminals on the matrix (with the
-// FP64 re-score of near ties in the FP32 mode); the Lance-Williams update of
-// the matrix after the round's merges (before the compaction)
-int64_t dense_default(int d);
+// dense phase (hac_dense.cu): room for the matrix of K clusters (allocated if
+// need be); whether this round should run on the matrix (entering it if
+// needed); the nearest-neighbour search of the round's terminals on the matrix
+// (with the FP64 re-score of near ties in the FP32 mode); the matrix after the
+// round's merges (after the compaction, Kold clusters before); every remaining
+// round in one launch, at most `limit` of them (0 = all)
+int64_t dense_default(int64_t n, int d, int linkage, int prec);
+int dense_reserve(hac_ctx *h, int K);
 int dense_maybe_enter(hac_ctx *h, cudaStream_t st, int K, RoundCtl &ctl);
 int dense_search(hac_ctx *h, cudaStream_t st, int K, int nterm, RoundCtl &ctl);
-int dense_update(hac_ctx *h, cudaStream_t st, int round, int K, int npairs);
+int dense_update(hac_ctx *h, cudaStream_t st, int round, int Kold, int K);
+int dense_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64_t limit,
+                 Counters *c);
+
+// points moved so that every cluster is one segment again, if they are not
+int relayout_if_stale(hac_ctx *h, cudaStream_t st);
+
+// one thread-block cluster of nct blocks (1 .. 16, a power of two; fewer if the
+// device cannot place them) running kern(*args) on st
+int launch_cluster(const void *kern, int nct, int threads, size_t smem, void *args,
+                   cudaStream_t st);
 
 }  // namespace hacg

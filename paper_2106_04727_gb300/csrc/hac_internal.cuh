@@ -176,28 +176,27 @@ struct State {
   int32_t *tinfo;       // node count of every level, then TI_TOP, TI_FIXED
   int32_t lvl_base[MAXLEV + 1];
   int32_t chb[MAXLEV + 1];
-  // dense phase (average linkage, one instance): once the active clusters
-  // fit, the whole matrix of their pair distances (the Section 5 cache with
-  // room for every pair), filled by one all-pairs sweep of the points and
-  // updated by Lance-Williams after every round.  Each entry is kept as the
-  // exact sum of its point distances (128-bit fixed point, so a merge adds
-  // sums exactly) and as the mean distance that sum gives (FP64); in the FP32
-  // mode an FP32-derived estimate carries the sign bit of the mean (its
-  // magnitude is the estimate) and the top bit of the sum.
+  // dense phase (average and complete linkage, one instance): the whole matrix
+  // of the active clusters' pair distances (the Section 5 cache with room for
+  // every pair), indexed by position in the active order and written anew over
+  // the compacted order after every round's merges.  Average: each entry is
+  // kept as the exact sum of its point distances (128-bit fixed point, so a
+  // merge adds sums exactly) and as the mean distance that sum gives (FP64);
+  // complete: as the distance.  In the FP32 mode an FP32-derived estimate
+  // carries the sign bit of the mean or distance (its magnitude is the
+  // estimate) and the top bit of the sum.
   int dense;            // 1 once the instance runs on the matrix
-  int dk;               // matrix dimension: active clusters at the switch
+  int dk, dld;          // matrix dimension (active clusters) and row stride
   int dexp;             // exponent of the fixed-point unit of the sweep sums
   int dsk;              // the FP32 sweep scales coordinates by 2^dsk
-  double dsl, dsh;      // 2^dexp and 2^(64 + dexp): a sum's low and high word scales
   double *dinv;         // 1 / size of the cluster at each matrix index
-  double *dmat;         // dk x dk, row-major; diagonal +inf
-  unsigned long long *dsum;  // 128-bit fixed-point sums of point distances of the
-                             // pairs i < j, packed upper triangle (four limb words
-                             // per pair; the top bit of the last marks an estimate)
-  int32_t *dq;          // this round: matrix index of each active position
-  uint8_t *dqm;         // after the merges: 1 if that cluster merged this round
-  int32_t *didx;        // cid -> matrix index (the cid's position at the switch)
-  int32_t *dcid;        // matrix index -> cid
+  double *dmat;         // dk rows of stride dld; diagonal +inf
+  double *dmat2;        // complete: the next round's matrix
+  // 128-bit fixed-point sums of point distances of the pairs i < j, packed
+  // upper triangle (two words per pair; the top bit of the second marks an
+  // estimate), and the next round's
+  unsigned long long *dsum, *dsum2;
+  int32_t *dma, *dmb;   // old positions of a new position's cluster and its partner
   int drq_cap;          // FP64 re-score queue (pairs, lower index first)
   int32_t *drq_a, *drq_b, *drq_pre;
   unsigned long long *drq_acc;  // fixed-point sums, two words per pair
@@ -328,6 +327,13 @@ __host__ __device__ inline int fin_cap(int d) {
   const int c = FIN_SMEM / fin_record_bytes(fin_dim(d)) & ~31;
   return c < FIN_MAX_K ? c : FIN_MAX_K;
 }
+
+// The same for rounds on the dense matrix (hac_dense.cu): at most DFIN_K active
+// clusters, one list entry per thread of a block.
+#ifndef HAC_DFIN_K
+#define HAC_DFIN_K 1024
+#endif
+constexpr int DFIN_K = HAC_DFIN_K;
 
 // tinfo entries after the per-level node counts
 constexpr int TI_TOP = MAXLEV + 1;    // lowest level with at most 32 nodes (the root's children)
