@@ -1616,6 +1616,9 @@ void fill_query_args(hac_ctx *h, QueryArgs &qa, int round, int K, int nterm) {
 bool use_brute(const hac_ctx *h) {
   const State &s = h->s;
   if (!closed_form(s.linkage) || s.prec != HAC_PREC_F32_RECHECK || s.max_inst != 1) return false;
+  // the screening's FP32 squares neither flush nor overflow
+  if (!(s.coord_scale >= (float)FIN_SCALE_LO && s.coord_scale < (float)FIN_SCALE_HI)) return false;
+  if (!h->own) return false;  // hac_run_static: no memory for the lists
   if (h->brute_env >= 0) return h->brute_env == 1 && (s.dp == 8 || s.dp == 16);
   return s.dp == 16;
 }
@@ -1662,6 +1665,13 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
   if (brute) {
     CK(cudaMemsetAsync(&s.ctr->npend, 0, sizeof(int32_t), st));
     qa.pend_out = s.blist;
+    if (!s.glist &&  // sized once per handle
+        ((rc = dalloc(h, &s.gu, h->n)) || (rc = dalloc(h, &s.gcnt, h->n)) ||
+         (rc = dalloc(h, &s.glist, (size_t)h->n * GRAM_LIST))))
+      return rc;
+    qa.gu = s.gu;
+    qa.gcnt = s.gcnt;
+    qa.glist = s.glist;
   }
   if (!dense && use_cand_avg(h)) {
     if (!s.lpos) {  // sized once per handle: BL_CAP positions per cluster
@@ -1683,7 +1693,8 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
     if (rc) return rc;
     ++ctl.dense_rounds;
   } else if (brute) {
-    CK(launch_brute(qa, s.dp, st));
+    CK(launch_brute(qa, s.dp, device_sms(), st));
+    h->launches += 3;
   } else {
     CK(launch_query(qa, s.dp, query_prec(s), st));
   }

@@ -156,6 +156,9 @@ struct State {
   // candidate lists of the exhaustive scan for average linkage (by position)
   int32_t *lpos, *lcnt;
   float *llb, *lub;
+  // exhaustive search of the closed-form linkages (by terminal)
+  float *gu;
+  int32_t *gcnt, *glist;
   int32_t *pair_lo, *pair_hi;
   double *pair_key;
   // dendrogram records
@@ -262,6 +265,9 @@ struct QueryArgs {
   int lcap;
   const int32_t *lpos, *lcnt;
   const float *lub;
+  // exhaustive search: U, candidates listed and their positions by terminal
+  float *gu;
+  int32_t *gcnt, *glist;
 };
 
 // pairs of at least this many point pairs are evaluated by the whole GPU
@@ -342,10 +348,11 @@ constexpr int TI_SIZE = MAXLEV + 3;
 
 // launches the nearest-neighbour query of every terminal (hac_query.cu)
 cudaError_t launch_query(const QueryArgs &a, int dp, int prec, cudaStream_t s);
-// the same search done exhaustively with tiles of cluster records staged in
-// shared memory (hac_brute.cu): closed-form linkages, FP32 + FP64 re-score,
+// the same search done exhaustively, screened by tensor-core products of the
+// cluster records (hac_brute.cu): closed-form linkages, FP32 + FP64 re-score,
 // one instance; uses pend_out (nterm entries) and ctr->npend (zeroed first)
-cudaError_t launch_brute(const QueryArgs &a, int dp, cudaStream_t s);
+cudaError_t launch_brute(const QueryArgs &a, int dp, int sms, cudaStream_t s);
+constexpr int GRAM_LIST = 48;  // candidates its screening lists per terminal
 // candidate lists for average linkage: every terminal scans every active
 // cluster's record (tiles in shared memory) and lists, by position, those
 // whose centroid lower bound is within its least Jensen upper bound
