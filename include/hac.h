@@ -226,7 +226,8 @@ const char *hac_strerror(int code);
  * loads the library holds until the process exits.  No cudaMalloc, cudaFree
  * or other allocating call is made.  The pair-distance cache needs memory, so
  * opts->cache_slots is ignored (no cache, hence no GPU-wide big-pair
- * evaluation), and the HAC_* environment overrides that hac_create reads
+ * evaluation; in HAC_PREC_F64 complete and average linkage move to a packed
+ * triangle of pair distances once it fits what is left of the array), and the HAC_* environment overrides that hac_create reads
  * (HAC_BIG_PAIRS, HAC_BIG_PAIRS_F64, HAC_WARP_BUDGET, HAC_BRUTE, HAC_DENSE_K) do
  * not apply;
  * these change speed only, never the result.  HAC_FLAG_NO_PRUNE is honoured.

@@ -1406,7 +1406,11 @@ int init_layout(hac_ctx *h, cudaStream_t st) {
   k_inst_set<<<1, 1, 0, st>>>(s, 0, (float)s.abs_slack, s.coord_scale, s.delta_pts, 0, (int)n, 0);
   k_morton<T><<<grid_for(n, TPB), TPB, 0, st>>>(X, n, d, mp, h->keys[0], h->vals[0]);
   CK(cudaGetLastError());
-  int sc = radix_sort(h, (int)n, mp.bits * d, st);
+  // a run that never searches the tree needs no spatial order; at few points
+  // its locality is worth less than the sort's 40 launches
+  const bool tree = !h->dense_first && !(h->tri && n <= h->tri_cap);
+  int sc = 0;
+  if (tree || n > FIN_MAX_K) sc = radix_sort(h, (int)n, mp.bits * d, st);
   if (sc < 0) return sc;
   h->ocur = h->pcur = 0;
   h->lay_n = n;
@@ -1420,8 +1424,7 @@ int init_layout(hac_ctx *h, cudaStream_t st) {
   c.nterm = (int)n;
   c.nactive = (int)n;
   CK(cudaMemcpyAsync(s.ctr, &c, sizeof(Counters), cudaMemcpyHostToDevice, st));
-  // (a run that starts on the dense matrix never searches the tree)
-  return h->dense_first ? HAC_OK : build_tree(h, s.order[0], (int)n, st);
+  return tree ? build_tree(h, s.order[0], (int)n, st) : HAC_OK;
 }
 
 // Canonical order of the merge records on the device, (height, size, cid_a)
@@ -1431,6 +1434,10 @@ int sort_records(hac_ctx *h, cudaStream_t st, hac_merge *out, int32_t *out_round
   State &s = h->s;
   const int64_t m = h->n - 1;
   if (m <= 0) return HAC_OK;
+  if (m <= FIN_MAX_K) {
+    h->launches += 1;
+    return launch_rec_sort(s, (int)m, out, out_round, st);
+  }
   const int mm = (int)m;
   const int g = grid_for(mm, TPB);
   int32_t *perm = nullptr;
@@ -1933,6 +1940,17 @@ int run_rounds(hac_ctx *h, const hac_opts &opt, cudaStream_t st, RoundCtl &ctl, 
       }
       K = c.nactive;
       nterm = c.nterm;
+      round += c.fin_rounds;
+      ctl.searches += c.fin_searches;
+      ctl.naive += c.fin_naive;
+      *rounds_out = round;
+      continue;
+    }
+    if (h->tri && K <= h->tri_cap) {
+      rc = tri_finish(h, st, K, nterm, round, &c);
+      if (rc) return rc;
+      if ((c.err & ~ERR_NONFINITE) || c.nactive != 1) return HAC_EINTERNAL;
+      K = 1;
       round += c.fin_rounds;
       ctl.searches += c.fin_searches;
       ctl.naive += c.fin_naive;
@@ -2516,6 +2534,18 @@ extern "C" int hac_run_static(const void *dev_points, int64_t n, int d, hac_dtyp
   h.dense_k = 0;  // the fixed array has no room for the dense matrix
   Carver cv{arena, 0, kStaticArenaBytes, true};
   if (!carve_state(h, cv)) return HAC_EINVAL;
+  // FP64 average / complete: the rest of the array holds the packed triangle of
+  // pair distances as soon as the active clusters' fits (not under a limit,
+  // which is checked between rounds)
+  if (!closed_form(h.s.linkage) && h.s.prec == HAC_PREC_F64 && !h.s.noprune && !opt.max_rounds &&
+      !(opt.timeout_s > 0)) {
+    const size_t at = (cv.off + 255) & ~(size_t)255;
+    const size_t cells = at < cv.cap ? (cv.cap - at) / sizeof(double) : 0;
+    int k = TRI_MAX_K;
+    while (k > 1 && (size_t)k * (k - 1) / 2 > cells) --k;
+    h.tri = (double *)(cv.base + at);
+    h.tri_cap = k;
+  }
   const cudaStream_t st = (cudaStream_t)opt.stream;
   rc = abi_guard([&] { return static_run(h, opt, st, dev_out); });
   if (rc == HAC_EDEVICE) cudaGetLastError();

@@ -1381,6 +1381,248 @@ __global__ void __launch_bounds__(DF_T, 1) k_dense_finish(DFinArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// FP64 rounds on a packed triangle (hac_run_static)
+// ---------------------------------------------------------------------------
+// The allocation-free entry point has a few MB to spare: once the active
+// clusters' packed upper triangle fits (8 B per pair: the sum of point
+// distances for average, the distance for complete), the FP64 mode fills it
+// from the points over the whole GPU and runs every remaining round in one
+// launch.  Without a cache its searches evaluate each big pair again in every
+// round, in one warp, and FP64 point pairs are bound by the SM's two-lane FP64
+// pipe: 1,024 points of 2-D average took 17.9 ms so, 0.68 here.
+// Entries are patched in place: a round's survivors add (or take the larger
+// of) their partners' entries.
+
+// one warp per pair of clusters
+template <int LK, int DP>
+__global__ void __launch_bounds__(256) k_tri_fill(State s, const int32_t *order, int K, int cur,
+                                                  double *tri_) {
+  const int lane = threadIdx.x & 31;
+  const long long cells = (long long)K * (K - 1) / 2;
+  const double *P = s.p64[cur];
+  const int32_t *seg = s.seg[cur];
+  unsigned long long pp = 0;
+  const bool single = K == (int)s.n;  // one thread per pair
+  const long long step = (long long)gridDim.x * blockDim.x >> (single ? 0 : 5);
+  for (long long t = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> (single ? 0 : 5);
+       t < cells; t += step) {
+    // column j of the triangle enumerated by columns: t = j (j - 1) / 2 + i
+    long long i, j;
+    tile_of(t, i, j);
+    ++j;
+    const int A = order[i], B = order[j];
+    int na = single ? 1 : s.csize[A], nb = single ? 1 : s.csize[B], sa = seg[A], sb = seg[B];
+    if (nb > na) {
+      int x = na;
+      na = nb;
+      nb = x;
+      x = sa;
+      sa = sb;
+      sb = x;
+    }
+    double acc = 0.0;
+    for (int u = single ? 0 : lane; u < na; u += 32) {
+      double x[DP];
+#pragma unroll
+      for (int k = 0; k < DP; ++k) x[k] = P[(size_t)(sa + u) * DP + k];
+      for (int v = 0; v < nb; ++v) {
+        double d2 = 0.0;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) {
+          if (k < s.d) {
+            const double e = x[k] - P[(size_t)(sb + v) * DP + k];
+            d2 = fma(e, e, d2);
+          }
+        }
+        if (LK == LK_COMPLETE)
+          acc = fmax(acc, d2);
+        else
+          acc += sqrt(d2);
+      }
+    }
+    if (!single) {
+      for (int o = 16; o; o >>= 1) {
+        const double y = __shfl_xor_sync(0xffffffffu, acc, o);
+        acc = LK == LK_COMPLETE ? fmax(acc, y) : acc + y;
+      }
+    }
+    if (single || lane == 0) {
+      tri_[tri(i, j, K)] = LK == LK_COMPLETE ? sqrt(acc) : acc;
+      pp += (unsigned long long)na * nb;
+    }
+  }
+  for (int o = 16; o; o >>= 1) pp += __shfl_xor_sync(0xffffffffu, pp, o);
+  if (lane == 0 && pp) atomicAdd(&s.ctr->point_pairs, pp);
+}
+
+struct TriArgs {
+  State s;
+  int K, nterm, round;
+  const int32_t *order;
+  double *tri;
+};
+
+constexpr int TRI_PER = (TRI_MAX_K + DF_T - 1) / DF_T;
+
+template <int LK>
+__global__ void __launch_bounds__(DF_T, 1) k_tri_finish(TriArgs a) {
+  // by position in the active list: cid, slot (position at the start); by slot:
+  // 1 / size and the partner of this round's merge (-1 none, -2 retired now)
+  __shared__ int s_cid[TRI_MAX_K], s_slot[TRI_MAX_K], s_term[TRI_MAX_K], s_part[TRI_MAX_K];
+  __shared__ double s_inv[TRI_MAX_K];
+  __shared__ int ws[DF_W];
+  const State &s = a.s;
+  const int rank = df_rank(), nct = df_count(), K0 = a.K;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int K = a.K, nterm = a.nterm, round = a.round;
+  double *T = a.tri;
+  for (int p = threadIdx.x; p < K; p += DF_T) {
+    const int c = a.order[p];
+    s_cid[p] = c;
+    s_slot[p] = p;
+    s_inv[p] = 1.0 / (double)s.csize[c];
+  }
+  for (int t = threadIdx.x; t < nterm; t += DF_T) s_term[t] = s.pos[s.term[t]];
+  __syncthreads();
+  auto at = [&](int x, int y) -> size_t { return x < y ? tri(x, y, K0) : tri(y, x, K0); };
+  long long searches = 0, naive = 0;
+  while (K > 1) {
+    searches += nterm;
+    naive += (long long)nterm * (K - 1);
+    for (int t = rank * DF_W + wid; t < nterm; t += nct * DF_W) {
+      const int self = s_term[t], q = s_slot[self], ci = s_cid[self];
+      const double iq = s_inv[q];
+      unsigned long long bk = KINF_D;
+      int bp = -1;
+#pragma unroll 4
+      for (int p = lane; p < K; p += 32) {
+        const int r = s_slot[p];
+        double v = p == self ? 0.0 : __ldcg(T + at(q, r));
+        // mean: 1 / size of the lower slot first, so both sides agree
+        if (LK == LK_AVERAGE) v = q < r ? v * iq * s_inv[r] : v * s_inv[r] * iq;
+        const unsigned long long k = (unsigned long long)__double_as_longlong(v);
+        if (p != self && (k < bk || (k == bk && bp >= 0 && s_cid[p] < s_cid[bp]))) {
+          bk = k;
+          bp = p;
+        }
+      }
+      int bc = bp >= 0 ? s_cid[bp] : INT_MAX;
+      warp_argmin_kc(bk, bc);
+      if (lane == 0) {
+        s.Ekey[ci] = __longlong_as_double((long long)bk);
+        s.Ecid[ci] = bc == INT_MAX ? -1 : bc;
+        if (bc == INT_MAX) atomicOr(&s.ctr->err, ERR_NO_NN);
+      }
+    }
+    df_sync();
+    for (int t = rank * DF_T + threadIdx.x; t < nterm; t += nct * DF_T) {
+      const int i = s_cid[s_term[t]];
+      const int j = __ldcg(&s.Ecid[i]);
+      if (j >= 0) s.succ[i] = j;
+    }
+    df_sync();
+    for (int t = rank * DF_T + threadIdx.x; t < nterm; t += nct * DF_T) {
+      const int i = s_cid[s_term[t]];
+      const int j = __ldcg(&s.Ecid[i]);
+      if (j < 0 || __ldcg(&s.succ[j]) != i || !(i < j || __ldcg(&s.isterm[j]) != round)) continue;
+      const int lo = min(i, j), hi = max(i, j);
+      const int sz = __ldcg(&s.csize[lo]) + __ldcg(&s.csize[hi]);
+      const int r = s.irec[0] + atomicAdd(&s.irecn[0], 1);
+      s.m_a[r] = lo;
+      s.m_b[r] = hi;
+      s.m_h[r] = __ldcg(&s.Ekey[i]);
+      s.m_size[r] = sz;
+      s.m_round[r] = round;
+      s.csize[lo] = sz;
+      s.succ[lo] = -1;
+      s.mround[lo] = round;
+      s.mround[hi] = round;
+      s.alive[hi] = 0;
+      s.partner[lo] = hi;
+    }
+    df_sync();
+    // chain repair and compaction, the same in every block
+    int c[TRI_PER], sl[TRI_PER], f[TRI_PER], cnt = 0;
+#pragma unroll
+    for (int r = 0; r < TRI_PER; ++r) {
+      const int p = threadIdx.x * TRI_PER + r;
+      c[r] = p < K ? s_cid[p] : -1;
+      sl[r] = p < K ? s_slot[p] : 0;
+      f[r] = 0;
+      if (c[r] >= 0) {
+        int part = -1;
+        if (__ldcg(&s.alive[c[r]])) {
+          int sc = __ldcg(&s.succ[c[r]]);
+          if (sc >= 0 && __ldcg(&s.mround[sc]) == round) {
+            sc = -1;
+            if (rank == 0) s.succ[c[r]] = -1;
+          }
+          // a retired cid's pos still is its slot: positions are not rewritten here
+          if (__ldcg(&s.mround[c[r]]) == round) part = s.pos[__ldcg(&s.partner[c[r]])];
+          f[r] = 1 | (sc < 0 ? 1 << 16 : 0);
+        }
+        s_part[sl[r]] = part;
+      }
+      cnt += f[r];
+    }
+    int tot;
+    int pre = df_scan(cnt, &tot, ws);
+    const int K2 = tot & 0xffff;
+    if (K2 >= K) {  // no pair merged: cannot happen
+      if (rank == 0 && threadIdx.x == 0) atomicOr(&s.ctr->err, ERR_NO_NN);
+      break;
+    }
+#pragma unroll
+    for (int r = 0; r < TRI_PER; ++r) {
+      if (f[r]) {
+        const int q = pre & 0xffff;
+        s_cid[q] = c[r];
+        s_slot[q] = sl[r];
+        s_inv[sl[r]] = 1.0 / (double)__ldcg(&s.csize[c[r]]);
+        if (f[r] >> 16) {
+          s_term[pre >> 16] = q;
+          if (rank == 0) s.isterm[c[r]] = round + 1;
+        }
+      }
+      pre += f[r];
+    }
+    __syncthreads();
+    // entries of the survivors: a warp per merged cluster and 32 others
+    const int segs = (K2 + 31) >> 5;
+    for (int t = rank * DF_W + wid; t < K2 * segs; t += nct * DF_W) {
+      const int x = s_slot[t / segs], b = s_part[x];
+      if (b < 0) continue;  // did not merge (uniform over the warp)
+      const int p = (t % segs) * 32 + lane;
+      if (p >= K2) continue;
+      const int y = s_slot[p], d = s_part[y];
+      if (y == x || (d >= 0 && y < x)) continue;  // both merged: the lower slot's warp does it
+      double v = __ldcg(T + at(x, y)), u = __ldcg(T + at(b, y));
+      v = LK == LK_COMPLETE ? fmax(v, u) : v + u;
+      if (d >= 0) {
+        const double g = __ldcg(T + at(x, d)), h = __ldcg(T + at(b, d));
+        u = LK == LK_COMPLETE ? fmax(g, h) : g + h;
+        v = LK == LK_COMPLETE ? fmax(v, u) : v + u;
+      }
+      T[at(x, y)] = v;
+    }
+    K = K2;
+    nterm = tot >> 16;
+    ++round;
+    df_sync();
+  }
+  if (rank != 0 || threadIdx.x != 0) return;
+  s.ctr->nactive = K;
+  s.ctr->nterm = nterm;
+  s.ctr->nmerges += a.K - K;
+  s.ctr->ltests += (unsigned long long)naive;
+  s.ctr->fin_rounds = round - a.round;
+  s.ctr->fin_searches = searches;
+  s.ctr->fin_naive = naive;
+  s.idone[0] = K <= 1;
+  s.iact[0] = K;
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 template <typename F>
@@ -1809,6 +2051,42 @@ int dense_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64
     s.dk = c->nactive;
     s.dld = dense_ld(c->nactive);
   }
+  return HAC_OK;
+}
+
+// Every remaining round of an FP64 run on the packed triangle at h->tri
+// (room for h->tri_cap clusters); the counters come back in *c.
+int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, Counters *c) {
+  State &s = h->s;
+  const int32_t *order = s.order[h->ocur];
+  const int g = device_sms() * 8;
+  const bool comp = s.linkage == LK_COMPLETE;
+#define TRI_FILL(DP)                                                                      \
+  (comp ? k_tri_fill<LK_COMPLETE, DP><<<g, 256, 0, st>>>(s, order, K, h->pcur, h->tri)    \
+        : k_tri_fill<LK_AVERAGE, DP><<<g, 256, 0, st>>>(s, order, K, h->pcur, h->tri))
+  switch (s.dp) {
+    case 2: TRI_FILL(2); break;
+    case 4: TRI_FILL(4); break;
+    case 8: TRI_FILL(8); break;
+    default: TRI_FILL(16);
+  }
+#undef TRI_FILL
+  CK(cudaGetLastError());
+  TriArgs a{};
+  a.s = s;
+  a.K = K;
+  a.nterm = nterm;
+  a.round = round;
+  a.order = order;
+  a.tri = h->tri;
+  const int nct = K <= 64 ? 1 : K <= 200 ? 8 : 16;
+  int rc = launch_cluster(comp ? (const void *)k_tri_finish<LK_COMPLETE>
+                               : (const void *)k_tri_finish<LK_AVERAGE>,
+                          nct, DF_T, 0, &a, st);
+  if (rc) return rc;
+  h->launches += 2;
+  CK(cudaMemcpyAsync(c, s.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
   return HAC_OK;
 }
 

@@ -159,6 +159,9 @@ struct hac_ctx {
   bool done = false;
   int64_t n_merges = 0;
   hac_stats_t st{};
+  // hac_run_static: memory for the packed triangle of up to tri_cap clusters
+  double *tri = nullptr;
+  int tri_cap = 0;
   hac_merge *dout = nullptr;        // canonical dendrogram (device)
   int32_t *dout_round = nullptr;
 };
@@ -258,6 +261,8 @@ struct FinArgs {
   int n_rec;             // direct: records to write
 };
 int launch_finish(FinArgs &a, cudaStream_t st);
+// the canonical order of at most FIN_MAX_K merge records in one block
+int launch_rec_sort(const State &s, int m, hac_merge *out, int32_t *out_round, cudaStream_t st);
 
 int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCtl &ctl,
                int *npairs_out);
@@ -284,6 +289,9 @@ int dense_search(hac_ctx *h, cudaStream_t st, int K, int nterm, RoundCtl &ctl);
 int dense_update(hac_ctx *h, cudaStream_t st, int round, int Kold, int K);
 int dense_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64_t limit,
                  Counters *c);
+
+// FP64 average / complete: every remaining round on the packed triangle
+int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, Counters *c);
 
 // points moved so that every cluster is one segment again, if they are not
 int relayout_if_stale(hac_ctx *h, cudaStream_t st);

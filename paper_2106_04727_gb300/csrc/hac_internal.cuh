@@ -340,6 +340,8 @@ __host__ __device__ inline int fin_cap(int d) {
 #define HAC_DFIN_K 1024
 #endif
 constexpr int DFIN_K = HAC_DFIN_K;
+// FP64 rounds on a packed triangle (hac_run_static's spare memory)
+constexpr int TRI_MAX_K = 1280;
 
 // tinfo entries after the per-level node counts
 constexpr int TI_TOP = MAXLEV + 1;    // lowest level with at most 32 nodes (the root's children)
