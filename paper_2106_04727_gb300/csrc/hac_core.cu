@@ -262,7 +262,7 @@ __global__ void k_layout(State s, const T *X, const int32_t *perm, const uint64_
     }
     s.csq[i] = sq;
     s.sse[i] = 0.0;
-    s.qvar[p] = 0.f;
+    s.qvar[p] = s.linkage == LK_WARD ? 1.f : 0.f;
     s.qsz[p] = 1;
     s.qseg[p] = (int32_t)p;
     s.plab[0][p] = i;
@@ -1028,6 +1028,7 @@ __global__ void k_cmp_top(State s, int nb) {
 // rounded up (the search's FP32 error bound covers the difference).
 __device__ float cluster_var_up(const State &s, int c, int sz) {
   if (s.linkage == LK_AVG2) return __double2float_ru(s.sse[c] / (double)sz);
+  if (s.linkage == LK_WARD) return 1.f / (float)sz;
   if (s.linkage != LK_AVERAGE) return 0.f;
   const int dp = s.dp;
   const double inv = 1.0 / (double)sz;
@@ -1073,7 +1074,7 @@ __global__ void k_cmp_write(State s, const int32_t *order, int32_t *order_out, i
       }
       s.qsz[ok] = sz;
       s.qseg[ok] = os;
-      s.qvar[ok] = sz > 1 ? cluster_var_up(s, c, sz) : 0.f;
+      s.qvar[ok] = sz > 1 ? cluster_var_up(s, c, sz) : s.linkage == LK_WARD ? 1.f : 0.f;
       s.qinst[ok] = s.iseq[s.inst[c]];
     }
     if (ist) {
@@ -1630,6 +1631,15 @@ bool use_brute(const hac_ctx *h) {
   return s.dp == 16;
 }
 
+// Searches for groups of terminals (hac_gsearch.cu): the closed-form linkages in
+// d <= 8, one instance, unless the ablation wants every cluster scanned or the
+// FP32 squares could flush or overflow.
+bool use_gsearch(const hac_ctx *h) {
+  const State &s = h->s;
+  return closed_form(s.linkage) && s.max_inst == 1 && !s.noprune && s.d <= 8 &&
+         s.coord_scale >= (float)FIN_SCALE_LO && s.coord_scale < (float)FIN_SCALE_HI;
+}
+
 // Candidate lists from the exhaustive scan instead of the tree for average
 // linkage in d > 8 (one instance); HAC_BRUTE=0 / 1 turns them off / on for any
 // row stride of 8 or 16.
@@ -1702,6 +1712,15 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
   } else if (brute) {
     CK(launch_brute(qa, s.dp, device_sms(), st));
     h->launches += 3;
+  } else if (use_gsearch(h)) {
+    CK(cudaMemsetAsync(&s.ctr->npend, 0, sizeof(int32_t), st));
+    qa.pend_out = s.blist;
+    CK(launch_gsearch(qa, st));
+    QueryArgs rest = qa;  // the near ties it left undecided
+    rest.term = s.blist;
+    rest.nterm_dev = &s.ctr->npend;
+    CK(launch_query(rest, s.dp, query_prec(s), st));
+    h->launches += 1;
   } else {
     CK(launch_query(qa, s.dp, query_prec(s), st));
   }

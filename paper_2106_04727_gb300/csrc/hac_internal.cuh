@@ -148,7 +148,8 @@ struct State {
   float *q32, *qblo, *qbhi;  // FP32 centroid and box, K x dp
   double *q64;               // FP64 centroid, K x dp
   int32_t *qsz, *qseg;       // size and segment start
-  float *qvar;               // variance (mean squared distance to the centroid), rounded up
+  float *qvar;               // variance (mean squared distance to the centroid), rounded
+                             // up; Ward: 1 / size
   // lists
   int32_t *order[2];    // active cids in spatial order
   int32_t *term;        // terminal cids
@@ -268,6 +269,7 @@ struct QueryArgs {
   // exhaustive search: U, candidates listed and their positions by terminal
   float *gu;
   int32_t *gcnt, *glist;
+  const int32_t *nterm_dev;  // if set, the number of terminals is read here
 };
 
 // pairs of at least this many point pairs are evaluated by the whole GPU
@@ -350,6 +352,15 @@ constexpr int TI_SIZE = MAXLEV + 3;
 
 // launches the nearest-neighbour query of every terminal (hac_query.cu)
 cudaError_t launch_query(const QueryArgs &a, int dp, int prec, cudaStream_t s);
+// the same search for Ward / avg-2 with d <= 8, one instance, for groups of
+// terminals (hac_gsearch.cu): leaves undecided terminals in pend_out and
+// ctr->npend (zeroed first) to launch_query (nterm_dev = &ctr->npend)
+cudaError_t launch_gsearch(const QueryArgs &a, cudaStream_t s);
+#ifndef HAC_GS_WIDE
+#define HAC_GS_WIDE 40000
+#endif
+constexpr int GS_WIDE = HAC_GS_WIDE;  // terminals from which a group is 32 (else 8)
+
 // the same search done exhaustively, screened by tensor-core products of the
 // cluster records (hac_brute.cu): closed-form linkages, FP32 + FP64 re-score,
 // one instance; uses pend_out (nterm entries) and ctr->npend (zeroed first)

@@ -1161,7 +1161,8 @@ __global__ void __launch_bounds__(QWARPS * 32, qminb(LK)) k_query(QueryArgs a) {
   __shared__ int s_ti[TI_SIZE];
   for (int i = threadIdx.x; i < TI_SIZE; i += blockDim.x) s_ti[i] = a.tinfo[i];
   __syncthreads();
-  for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < a.nterm; t += nw) {
+  const int nterm = a.nterm_dev ? *a.nterm_dev : a.nterm;
+  for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < nterm; t += nw) {
     const int ci = a.term[t];
     const int own = a.pbkt[a.pos[ci]];
     // a candidate list from the exhaustive scan replaces the tree traversal
@@ -1238,6 +1239,7 @@ __global__ void __launch_bounds__(QWARPS * 32, qminb(LK)) k_query(QueryArgs a) {
 template <int LK, int PREC>
 cudaError_t launch_lk(const QueryArgs &a, int dp, cudaStream_t s) {
   int blocks = (a.nterm + QWARPS - 1) / QWARPS;
+  if (a.nterm_dev && blocks > 608) blocks = 608;  // few terminals expected: grid-stride
   if (blocks < 1) blocks = 1;
   switch (dp) {
     case 2: k_query<LK, 2, PREC><<<blocks, QWARPS * 32, 0, s>>>(a); break;

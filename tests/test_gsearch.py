@@ -1,0 +1,56 @@
+"""The grouped search of Ward and avg-2 (csrc/hac_gsearch.cu) in runs above the
+one-launch capacity: groups of 8 and, from 40,000 terminals, of 32, in every
+dimension it takes, ragged group and bucket ends, ties and near ties (left to
+the warp-per-terminal FP64 search)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2106_04727_gb300 import hac, inputs
+
+pytestmark = pytest.mark.gpu
+
+LKS = ["ward", "average_sq"]
+
+
+def _check(got, want, rtol=1e-9):
+    c = oracle.compare(got, want, rtol=rtol)
+    assert c["ok"], c
+    key = lambda t: sorted(zip(t["round"].tolist(), t["a"].tolist(), t["b"].tolist()))
+    assert key(got) == key(want)
+
+
+@pytest.mark.parametrize("lk", LKS)
+@pytest.mark.parametrize("d", list(range(1, 9)))
+def test_every_dimension(lk, d):
+    """n = 4,097 + 7 d: groups of 8 with a ragged last one."""
+    dt = np.float32 if d % 2 else np.float64
+    X = inputs.gaussian_mixture(4097 + 7 * d, d, 9, seed=50 + d, dtype=dt)
+    _check(hac.cluster(X, lk), oracle.rounds(X.astype(np.float64), lk))
+
+
+@pytest.mark.parametrize("lk", LKS)
+@pytest.mark.parametrize("name,n", [("gmm5d_1m_f32", 50_003), ("gaussiandisc2d_1m_f32", 70_001),
+                                    ("uniformfill5d_1m_f32", 41_000)])
+def test_wide_groups(lk, name, n):
+    """Groups of 32 in the first rounds, of 8 later."""
+    X = inputs.workload(name, n=n)
+    want = oracle.parchain_cpu(X.astype(np.float64), lk)
+    _check(hac.cluster(X, lk), want)
+
+
+@pytest.mark.parametrize("lk", LKS)
+@pytest.mark.parametrize("kind", ["lattice", "duplicates", "line", "outliers"])
+def test_hard_inputs(lk, kind):
+    """The same tree as with every cluster scanned in FP64 (no pruning, no
+    grouping)."""
+    if kind == "lattice":
+        X = inputs.lattice(5000, 2, seed=2, levels=40)
+    elif kind == "duplicates":
+        X = np.repeat(inputs.gaussian_mixture(450, 3, 5, seed=7), 10, axis=0)
+    elif kind == "line":
+        X = np.arange(4500, dtype=np.float32)[:, None] * np.float32(0.5)
+    else:
+        X = np.concatenate([1e-3 * inputs.gaussian_mixture(4600, 4, 6, seed=3),
+                            np.full((1, 4), 1e5, np.float32), np.full((1, 4), -3e4, np.float32)])
+    _check(hac.cluster(X, lk), hac.cluster(X, lk, no_prune=True), rtol=1e-12)
