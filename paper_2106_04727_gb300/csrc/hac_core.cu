@@ -230,58 +230,82 @@ __global__ void k_morton(const T *X, int64_t n, int d, MortonParams mp, uint64_t
   }
 }
 
+// The initial state in two sweeps.  What belongs to a cid (thread i = cid i)
+// comes from the input order, so its 20 arrays are written in rows of
+// consecutive threads; only what depends on the position (thread p) gathers a
+// point and scatters the three words that lead from a cid to its position.
+// One sweep over positions, which scattered everything, took 9.6 ms at 10^7
+// 2-D points (the whole initialisation 13.4 ms, 5.0 this way).  Points are kept only for the linkages that evaluate
+// point pairs, boxes only for complete linkage, squared norms for average.
 template <typename T>
-__global__ void k_layout(State s, const T *X, const int32_t *perm, const uint64_t *skey,
-                         MortonParams ctr_) {
+__global__ void k_layout_cid(State s, const T *X, MortonParams ctr_) {
   // ctr_.lo holds the recentring offset
   const int64_t n = s.n;
   const int d = s.d, dp = s.dp;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int i = perm[p];
-    for (int k = 0; k < dp; ++k) {
-      double x = k < d ? (double)X[(int64_t)i * d + k] - ctr_.lo[k] : 0.0;
-      s.p64[0][p * dp + k] = x;
-      // FP32 input stays unrounded (exact) in the FP32 copy; differences of
-      // FP32 numbers then carry only relative rounding error
-      s.p32[0][p * dp + k] = s.pts32_exact ? (k < d ? (float)X[(int64_t)i * d + k] : 0.f) : (float)x;
-      s.csum[(int64_t)i * dp + k] = x;
-      s.cent[(int64_t)i * dp + k] = x;
-      s.cent32[(int64_t)i * dp + k] = (float)x;
-      s.blo[(int64_t)i * dp + k] = __double2float_rd(x);
-      s.bhi[(int64_t)i * dp + k] = __double2float_ru(x);
-      s.q32[p * dp + k] = (float)x;
-      s.q64[p * dp + k] = x;
-      s.qblo[p * dp + k] = __double2float_rd(x);
-      s.qbhi[p * dp + k] = __double2float_ru(x);
-    }
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     double sq = 0.0;
-    for (int k = 0; k < d; ++k) {
-      const double x = (double)X[(int64_t)i * d + k] - ctr_.lo[k];
+    for (int k = 0; k < dp; ++k) {
+      const double x = k < d ? (double)X[i * d + k] - ctr_.lo[k] : 0.0;
+      s.csum[i * dp + k] = x;
+      s.cent[i * dp + k] = x;
+      s.cent32[i * dp + k] = (float)x;
+      if (s.linkage == LK_COMPLETE) {
+        s.blo[i * dp + k] = __double2float_rd(x);
+        s.bhi[i * dp + k] = __double2float_ru(x);
+      }
       sq += x * x;
     }
-    s.csq[i] = sq;
+    if (s.linkage == LK_AVERAGE) s.csq[i] = sq;
     s.sse[i] = 0.0;
-    s.qvar[p] = s.linkage == LK_WARD ? 1.f : 0.f;
-    s.qsz[p] = 1;
-    s.qseg[p] = (int32_t)p;
-    s.plab[0][p] = i;
-    s.seg[0][i] = (int32_t)p;
     s.csize[i] = 1;
     s.succ[i] = -1;
     s.pred[i] = PRED_EMPTY;
     s.mround[i] = -1;
     s.isterm[i] = 0;
     s.alive[i] = 1;
-    s.rootof[i] = i;
+    s.rootof[i] = (int32_t)i;
     s.reloff[i] = 0;
     s.gen[i] = 0;
     s.inst[i] = 0;
+  }
+}
+
+template <typename T>
+__global__ void k_layout_pos(State s, const T *X, const int32_t *perm, const uint64_t *skey,
+                             MortonParams ctr_) {
+  const int64_t n = s.n;
+  const int d = s.d, dp = s.dp;
+  const bool points = !closed_form(s.linkage);
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
+       p += (int64_t)gridDim.x * blockDim.x) {
+    const int i = perm[p];
+    for (int k = 0; k < dp; ++k) {
+      const double x = k < d ? (double)X[(int64_t)i * d + k] - ctr_.lo[k] : 0.0;
+      s.q32[p * dp + k] = (float)x;
+      s.q64[p * dp + k] = x;
+      if (points) {
+        s.p64[0][p * dp + k] = x;
+        // FP32 input stays unrounded (exact) in the FP32 copy; differences of
+        // FP32 numbers then carry only relative rounding error
+        s.p32[0][p * dp + k] =
+            s.pts32_exact ? (k < d ? (float)X[(int64_t)i * d + k] : 0.f) : (float)x;
+      }
+      if (s.linkage == LK_COMPLETE) {
+        s.qblo[p * dp + k] = __double2float_rd(x);
+        s.qbhi[p * dp + k] = __double2float_ru(x);
+      }
+    }
+    s.qvar[p] = s.linkage == LK_WARD ? 1.f : 0.f;
+    s.qsz[p] = 1;
+    s.qseg[p] = (int32_t)p;
+    s.plab[0][p] = i;
     s.qinst[p] = 0;
     s.order[0][p] = i;
+    s.term[p] = i;
+    s.seg[0][i] = (int32_t)p;
     s.pos[i] = (int32_t)p;
     s.mkey[i] = skey[p];
-    s.term[p] = i;
   }
 }
 
@@ -466,6 +490,7 @@ __device__ void tg_node_box(const State &s, int L, int j, int mb, int lane) {
     il = min(il, __shfl_xor_sync(0xffffffffu, il, o));
     ih = max(ih, __shfl_xor_sync(0xffffffffu, ih, o));
   }
+  const bool comp = s.linkage == LK_COMPLETE;  // the only one whose bounds use point boxes
   const int node = s.lvl_base[L] + j;
   if (lane == 0) {
     s.ninlo[node] = il;
@@ -478,25 +503,29 @@ __device__ void tg_node_box(const State &s, int L, int j, int mb, int lane) {
     if (L) {
       lo = v ? s.nclo[c * DP + k] : INFINITY;
       hi = v ? s.nchi[c * DP + k] : -INFINITY;
-      hm = v ? s.nhmin[c * DP + k] : INFINITY;
-      lm = v ? s.nlmax[c * DP + k] : -INFINITY;
+      hm = v && comp ? s.nhmin[c * DP + k] : INFINITY;
+      lm = v && comp ? s.nlmax[c * DP + k] : -INFINITY;
     } else {
       lo = v ? s.q32[c * DP + k] : INFINITY;
       hi = v ? s.q32[c * DP + k] : -INFINITY;
-      hm = v ? s.qbhi[c * DP + k] : INFINITY;
-      lm = v ? s.qblo[c * DP + k] : -INFINITY;
+      hm = v && comp ? s.qbhi[c * DP + k] : INFINITY;
+      lm = v && comp ? s.qblo[c * DP + k] : -INFINITY;
     }
     for (int o = 16; o; o >>= 1) {
       lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
       hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      hm = fminf(hm, __shfl_xor_sync(0xffffffffu, hm, o));
-      lm = fmaxf(lm, __shfl_xor_sync(0xffffffffu, lm, o));
+      if (comp) {
+        hm = fminf(hm, __shfl_xor_sync(0xffffffffu, hm, o));
+        lm = fmaxf(lm, __shfl_xor_sync(0xffffffffu, lm, o));
+      }
     }
     if (lane == k) {
       s.nclo[(size_t)node * DP + k] = lo;
       s.nchi[(size_t)node * DP + k] = hi;
-      s.nhmin[(size_t)node * DP + k] = hm;
-      s.nlmax[(size_t)node * DP + k] = lm;
+      if (comp) {
+        s.nhmin[(size_t)node * DP + k] = hm;
+        s.nlmax[(size_t)node * DP + k] = lm;
+      }
     }
   }
 }
@@ -666,14 +695,23 @@ __global__ void k_chain(State s, int nterm) {
   }
 }
 
-// parallel filter for reciprocal nearest neighbours: each pair once
+// parallel filter for reciprocal nearest neighbours: each pair once (one
+// counter addition per warp: additions to one address are served one by one)
 __global__ void k_rnn(State s, int nterm, int round) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nterm; t += gridDim.x * blockDim.x) {
-    const int i = s.term[t];
-    const int j = s.succ[i];
-    if (j < 0) continue;
-    if (s.succ[j] == i && (i < j || s.isterm[j] != round)) {
-      const int p = atomicAdd(&s.ctr->npairs, 1);
+  const int lane = threadIdx.x & 31;
+  for (int t0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; t0 < nterm;
+       t0 += gridDim.x * blockDim.x) {
+    const int t = t0 + lane;
+    const int i = t < nterm ? s.term[t] : -1;
+    const int j = i >= 0 ? s.succ[i] : -1;
+    const bool pair = j >= 0 && s.succ[j] == i && (i < j || s.isterm[j] != round);
+    const unsigned m = __ballot_sync(0xffffffffu, pair);
+    if (!m) continue;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&s.ctr->npairs, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (pair) {
+      const int p = base + __popc(m & ((1u << lane) - 1u));
       s.pair_lo[p] = min(i, j);
       s.pair_hi[p] = max(i, j);
       s.pair_key[p] = s.Ekey[i];
@@ -682,19 +720,33 @@ __global__ void k_rnn(State s, int nterm, int round) {
 }
 
 // merge every reciprocal pair: the cluster keeps the smaller cid
+// (record slots and the instance counters: one addition per warp and instance;
+// filter and merges of the first round of 10^7 2-D points, 3.1 * 10^6 pairs, took
+// 5.5 ms with one per pair, 2.6 this way and with boxes left to complete linkage)
 __global__ void k_merge(State s, int round, int npairs) {
   const int dp = s.dp;
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npairs; p += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  for (int p0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; p0 < npairs;
+       p0 += gridDim.x * blockDim.x) {
+    const int p = p0 + lane;
+    const unsigned act = __ballot_sync(0xffffffffu, p < npairs);
+    if (p >= npairs) continue;
     const int lo = s.pair_lo[p], hi = s.pair_hi[p];
     const double key = s.pair_key[p];
     const int na = s.csize[lo], nb = s.csize[hi];
     const int ins = s.inst[lo];
-    atomicAdd(&s.ctr->nmerges, 1);
-    const int m = s.irec[ins] + atomicAdd(&s.irecn[ins], 1);
-    if (atomicSub(&s.iact[ins], 1) == 2) {  // one cluster left
-      s.idone[ins] = 1;
-      s.done_list[atomicAdd(&s.ctr->ndone, 1)] = ins;
+    const unsigned same = __match_any_sync(act, ins);
+    const int lead = __ffs(same) - 1, cnt = __popc(same);
+    int m = 0;
+    if (lane == lead) {
+      atomicAdd(&s.ctr->nmerges, cnt);
+      m = s.irec[ins] + atomicAdd(&s.irecn[ins], cnt);
+      if (atomicSub(&s.iact[ins], cnt) - cnt == 1) {  // one cluster left
+        s.idone[ins] = 1;
+        s.done_list[atomicAdd(&s.ctr->ndone, 1)] = ins;
+      }
     }
+    m = __shfl_sync(same, m, lead) + __popc(same & ((1u << lane) - 1u));
     s.m_a[m] = lo;
     s.m_b[m] = hi;
     s.m_h[m] = s.linkage == LK_WARD ? sqrt(key) : key;
@@ -715,10 +767,12 @@ __global__ void k_merge(State s, int round, int npairs) {
       const double c = sum * inv;
       s.cent[(size_t)lo * dp + k] = c;
       s.cent32[(size_t)lo * dp + k] = (float)c;
-      s.blo[(size_t)lo * dp + k] = fminf(s.blo[(size_t)lo * dp + k], s.blo[(size_t)hi * dp + k]);
-      s.bhi[(size_t)lo * dp + k] = fmaxf(s.bhi[(size_t)lo * dp + k], s.bhi[(size_t)hi * dp + k]);
+      if (s.linkage == LK_COMPLETE) {
+        s.blo[(size_t)lo * dp + k] = fminf(s.blo[(size_t)lo * dp + k], s.blo[(size_t)hi * dp + k]);
+        s.bhi[(size_t)lo * dp + k] = fmaxf(s.bhi[(size_t)lo * dp + k], s.bhi[(size_t)hi * dp + k]);
+      }
     }
-    s.csq[lo] += s.csq[hi];
+    if (s.linkage == LK_AVERAGE) s.csq[lo] += s.csq[hi];
     s.csize[lo] = na + nb;
     s.succ[lo] = -1;
     s.pred[lo] = PRED_EMPTY;
@@ -1069,8 +1123,10 @@ __global__ void k_cmp_write(State s, const int32_t *order, int32_t *order_out, i
       for (int k = 0; k < dp; ++k) {
         s.q32[(size_t)ok * dp + k] = s.cent32[(size_t)c * dp + k];
         s.q64[(size_t)ok * dp + k] = s.cent[(size_t)c * dp + k];
-        s.qblo[(size_t)ok * dp + k] = s.blo[(size_t)c * dp + k];
-        s.qbhi[(size_t)ok * dp + k] = s.bhi[(size_t)c * dp + k];
+        if (s.linkage == LK_COMPLETE) {
+          s.qblo[(size_t)ok * dp + k] = s.blo[(size_t)c * dp + k];
+          s.qbhi[(size_t)ok * dp + k] = s.bhi[(size_t)c * dp + k];
+        }
       }
       s.qsz[ok] = sz;
       s.qseg[ok] = os;
@@ -1375,7 +1431,7 @@ int init_layout(hac_ctx *h, cudaStream_t st) {
   // counters start from zero (the allocation-free arena keeps the last call's)
   CK(cudaMemsetAsync(s.ctr, 0, sizeof(Counters), st));
   k_bbox<T><<<grid_for(n, TPB), TPB, 0, st>>>(X, n, d, h->bb, h->bb + MAXD, s.ctr);
-  h->launches += 3;  // bbox, morton, layout
+  h->launches += 4;  // bbox, morton, two layout sweeps
   CK(cudaGetLastError());
   Counters c0;
   CK(cudaMemcpyAsync(bb, h->bb, sizeof(bb), cudaMemcpyDeviceToHost, st));
@@ -1419,7 +1475,8 @@ int init_layout(hac_ctx *h, cudaStream_t st) {
   s.dense = 0;
   s.dk = 0;
   h->lay_stale = 0;
-  k_layout<T><<<grid_for(n, TPB), TPB, 0, st>>>(s, X, h->vals[sc], h->keys[sc], ctrp);
+  k_layout_cid<T><<<grid_for(n, TPB), TPB, 0, st>>>(s, X, ctrp);
+  k_layout_pos<T><<<grid_for(n, TPB), TPB, 0, st>>>(s, X, h->vals[sc], h->keys[sc], ctrp);
   CK(cudaGetLastError());
   Counters c{};
   c.nterm = (int)n;
