@@ -25,7 +25,9 @@
 // scans more records per terminal and fewer instructions per record.  Measured,
 // Ward whole runs of 10^6 points (ms, group size from GS_WIDE terminals on):
 // 2-D 17.0 / 17.2 / 17.2 (8 / 16 / 32), 5-D 45.6 / 47.4 / 54.3, 8-D 96.4 / 94.3 /
-// 107.9; the warp-per-terminal search: 27.6, 59.5, 170.  Below that few groups
+// 107.9; the warp-per-terminal search: 27.6, 59.5, 170.  10^7 2-D points have
+// enough terminals for the widest: first round 9.8 ms with 8, 4.2 with 32 (43
+// before).  Below that few groups
 // leave warps idle: 60,000 points in 5-D 7.5 with 4, 8.2 with 8 (9.8 before).
 // A terminal that reaches much farther than its group (a large cluster among
 // singletons: a node's bound knows only its smallest size) is searched by the
@@ -36,10 +38,13 @@ namespace hacg {
 
 namespace {
 
-// group sizes (from GS_WIDE terminals on, and below), how many binary orders of
+// group sizes (from GS_WIDE terminals on in d <= 2, above, and below), how many binary orders of
 // magnitude over its group's mean a squared radius may be, warps per block
 #ifndef HAC_GS_W
 #define HAC_GS_W 8
+#endif
+#ifndef HAC_GS_W2
+#define HAC_GS_W2 32
 #endif
 #ifndef HAC_GS_N
 #define HAC_GS_N 4
@@ -50,7 +55,7 @@ namespace {
 #ifndef HAC_GS_CUT
 #define HAC_GS_CUT 2
 #endif
-constexpr int GS_W = HAC_GS_W, GS_N = HAC_GS_N;
+constexpr int GS_W2 = HAC_GS_W2, GS_W = HAC_GS_W, GS_N = HAC_GS_N;
 constexpr int GW = HAC_GS_GW;         // warps per block
 constexpr int GSTK = 320;     // >= 32 + 31 * (MAXLEV) entries of a depth-first stack
 
@@ -369,12 +374,13 @@ __global__ void __launch_bounds__(GW * 32) k_gsearch(QueryArgs a) {
 template <int LK, int D>
 cudaError_t launch_g(const QueryArgs &a, cudaStream_t s) {
   constexpr int DP = D <= 2 ? 2 : D <= 4 ? 4 : 8;
+  constexpr int W = D <= 2 ? GS_W2 : GS_W;
   const bool wide = a.nterm >= GS_WIDE;
-  const int G = wide ? GS_W : GS_N;
+  const int G = wide ? W : GS_N;
   const int groups = (a.nterm + G - 1) / G;
   const int blocks = (groups + GW - 1) / GW;
   if (wide)
-    k_gsearch<LK, D, DP, GS_W><<<blocks, GW * 32, 0, s>>>(a);
+    k_gsearch<LK, D, DP, W><<<blocks, GW * 32, 0, s>>>(a);
   else
     k_gsearch<LK, D, DP, GS_N><<<blocks, GW * 32, 0, s>>>(a);
   return cudaGetLastError();
