@@ -1796,12 +1796,17 @@ int dense_alloc(hac_ctx *h, int64_t cap) {
   const int nbuf = s.linkage == LK_COMPLETE ? 2 : 3;
   int rc = dalloc(h, &h->dense_buf, nbuf * buf);
   if (rc) return rc;
-  if ((rc = dalloc(h, &s.dma, cap)) || (rc = dalloc(h, &s.dmb, cap)) ||
-      (rc = dalloc(h, &s.dinv, cap)) || (rc = dalloc(h, &s.drq_a, rqcap)) ||
-      (rc = dalloc(h, &s.drq_b, rqcap)) || (rc = dalloc(h, &s.drq_pre, rqcap + 1)) ||
-      (rc = dalloc(h, &s.drq_acc, LIMBS * (size_t)rqcap)) || (rc = dalloc(h, &s.dpend[0], cap)) ||
-      (rc = dalloc(h, &s.dpend[1], cap)))
-    return rc;
+  SlabAlloc m;
+  m.add(&s.dma, cap);
+  m.add(&s.dmb, cap);
+  m.add(&s.dinv, cap);
+  m.add(&s.drq_a, rqcap);
+  m.add(&s.drq_b, rqcap);
+  m.add(&s.drq_pre, rqcap + 1);
+  m.add(&s.drq_acc, LIMBS * (size_t)rqcap);
+  m.add(&s.dpend[0], cap);
+  m.add(&s.dpend[1], cap);
+  if ((rc = m.commit(h))) return rc;
   s.drq_cap = rqcap;
   h->dense_cap = cap;
   h->dense_stride = buf;

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <new>
 #include <vector>
@@ -186,6 +187,36 @@ int dalloc(hac_ctx *h, T **p, size_t count) {
   *p = (T *)q;
   return HAC_OK;
 }
+
+// Several arrays in one allocation: add() them all, then commit().  A handle
+// holds about 75; one cudaMalloc and cudaFree each made 0.45 ms of a 0.63 ms
+// hac.cluster of 64 points.
+struct SlabAlloc {
+  static constexpr int kMax = 96;
+  static constexpr size_t kAlign = 256;
+  void **at[kMax];
+  size_t off[kMax];
+  int n = 0;
+  size_t bytes = 0;
+  template <typename T>
+  void add(T **p, size_t count) {
+    if (n == kMax) {  // counted again by commit
+      ++n;
+      return;
+    }
+    at[n] = (void **)p;
+    off[n++] = bytes;
+    bytes += (std::max<size_t>(count, 1) * sizeof(T) + kAlign - 1) / kAlign * kAlign;
+  }
+  int commit(hac_ctx *h) {
+    if (n > kMax) return HAC_EINTERNAL;
+    unsigned char *q = nullptr;
+    const int rc = dalloc(h, &q, bytes);
+    if (rc) return rc;
+    for (int i = 0; i < n; ++i) *at[i] = q + off[i];
+    return HAC_OK;
+  }
+};
 
 // Runs f() and turns a C++ exception (a failed host allocation, a thread
 // that could not start) into a status code, so that none crosses the C ABI.

@@ -296,10 +296,11 @@ int engine_init(Engine &e, hac_linkage lk, int d, hac_dtype dt, int64_t cap, con
   int rc = alloc_state(&h);
   if (rc) return rc;
   const size_t esz = dt == HAC_F32 ? 4 : 8;
-  if ((rc = dalloc(&h, &e.stage, (size_t)cap * d * esz)) ||
-      (rc = dalloc(&h, &e.d_ai, (size_t)SRV_ADMIT_MAX)) ||
-      (rc = dalloc(&h, &e.d_rec, (size_t)cap)) || (rc = dalloc(&h, &e.d_fin, 2 * SRV_MAX_INST)))
-    return rc;
+  SlabAlloc m;
+  m.add(&e.stage, (size_t)cap * d * esz);
+  m.add(&e.d_ai, (size_t)SRV_ADMIT_MAX);
+  m.add(&e.d_rec, (size_t)cap);
+  m.add(&e.d_fin, 2 * SRV_MAX_INST);
   if (cudaMallocHost(&e.h_stage, (size_t)cap * d * esz) != cudaSuccess ||
       cudaMallocHost(&e.h_rec, (size_t)cap * sizeof(RecOut)) != cudaSuccess) {
     cudaGetLastError();
@@ -312,27 +313,38 @@ int engine_init(Engine &e, hac_linkage lk, int d, hac_dtype dt, int64_t cap, con
     const int64_t icap = std::max<int64_t>(4 * cap, 1 << 16);
     const int bcap = 1 << 18;
     const size_t per = (size_t)std::max(BIG_MAXT, cdiv(cap, BIG_TILE) + 1);
-    if ((rc = dalloc(&h, &s.ckey, cells)) || (rc = dalloc(&h, &s.cval, cells)) ||
-        (rc = dalloc(&h, &s.cerr, cells)) || (rc = dalloc(&h, &s.cpart, cells)) ||
-        (rc = dalloc(&h, &s.breq_base, bcap)) || (rc = dalloc(&h, &s.breq_cov, bcap)) ||
-        (rc = dalloc(&h, &s.breq_berr, bcap)) || (rc = dalloc(&h, &s.ins_i, icap)) ||
-        (rc = dalloc(&h, &s.ins_j, icap)) || (rc = dalloc(&h, &s.ins_v, icap)) ||
-        (rc = dalloc(&h, &s.ins_e, icap)) || (rc = dalloc(&h, &s.breq_i, bcap)) ||
-        (rc = dalloc(&h, &s.breq_j, bcap)) || (rc = dalloc(&h, &s.breq_sa, bcap)) ||
-        (rc = dalloc(&h, &s.breq_na, bcap)) || (rc = dalloc(&h, &s.breq_sb, bcap)) ||
-        (rc = dalloc(&h, &s.breq_nb, bcap)) || (rc = dalloc(&h, &s.breq_exact, bcap)) ||
-        (rc = dalloc(&h, &s.bsched, BS_SIZE)) ||
-        (rc = dalloc(&h, &s.bmax2, BIG_BATCH)) ||
-        (rc = dalloc(&h, &s.bpart, (size_t)BIG_BATCH * per)) ||
-        (rc = dalloc(&h, &s.pend[0], cap)) || (rc = dalloc(&h, &s.pend[1], cap)) ||
-        (rc = dalloc(&h, &s.side_key, 2 * bcap)) || (rc = dalloc(&h, &s.side_val, 2 * bcap)) ||
-        (rc = dalloc(&h, &s.side_err, 2 * bcap)))
-      return rc;
+    m.add(&s.ckey, cells);
+    m.add(&s.cval, cells);
+    m.add(&s.cerr, cells);
+    m.add(&s.cpart, cells);
+    m.add(&s.breq_base, bcap);
+    m.add(&s.breq_cov, bcap);
+    m.add(&s.breq_berr, bcap);
+    m.add(&s.ins_i, icap);
+    m.add(&s.ins_j, icap);
+    m.add(&s.ins_v, icap);
+    m.add(&s.ins_e, icap);
+    m.add(&s.breq_i, bcap);
+    m.add(&s.breq_j, bcap);
+    m.add(&s.breq_sa, bcap);
+    m.add(&s.breq_na, bcap);
+    m.add(&s.breq_sb, bcap);
+    m.add(&s.breq_nb, bcap);
+    m.add(&s.breq_exact, bcap);
+    m.add(&s.bsched, BS_SIZE);
+    m.add(&s.bmax2, BIG_BATCH);
+    m.add(&s.bpart, (size_t)BIG_BATCH * per);
+    m.add(&s.pend[0], cap);
+    m.add(&s.pend[1], cap);
+    m.add(&s.side_key, 2 * bcap);
+    m.add(&s.side_val, 2 * bcap);
+    m.add(&s.side_err, 2 * bcap);
     s.ins_cap = (int)icap;
     s.breq_cap = bcap;
     s.side_cap = 2 * bcap;
     h.cache_alloc_slots = slots;
   }
+  if ((rc = m.commit(&h))) return rc;
   s.cache_slots = slots;
   const cudaStream_t st = h.own;
   CK(cudaMemsetAsync(s.ctr, 0, sizeof(Counters), st));
