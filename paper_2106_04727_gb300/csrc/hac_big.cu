@@ -112,7 +112,10 @@ __device__ void cache_insert_evict(const State &s, int owner, int nbr, int nbr_g
         return;
       }
       if (slot_free(s, cur)) {
-        if (slot_put(s, base + t, cur, want, v, e)) return;
+        if (slot_put(s, base + t, cur, want, v, e)) {
+          s.cused[owner] = 1;
+          return;
+        }
         continue;
       }
       if (cur == CKEY_BUSY) continue;

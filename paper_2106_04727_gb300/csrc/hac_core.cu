@@ -862,6 +862,7 @@ __global__ void k_cache_merge(State s, int npairs, int round) {
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < npairs; p += warps) {
     const int lo = s.pair_lo[p], hi = s.pair_hi[p];
+    if (!s.cused[lo] && !s.cused[hi]) continue;  // both tables empty: so is the new one
     const double na = (double)s.osize[lo], nb = (double)s.osize[hi];
     if (lane == 0) cnt[wib][0] = cnt[wib][1] = cnt[wib][2] = cnt[wib][3] = 0;
     __syncwarp();
@@ -1010,7 +1011,10 @@ __global__ void k_cache_merge(State s, int npairs, int round) {
         s.ckey[slot] = CKEY_EMPTY;
       }
     }
-    if (lane == 0) atomicAdd((unsigned long long *)&s.ctr->cache_lw, (unsigned long long)nN);
+    if (lane == 0) {
+      s.cused[lo] = nN + nQ > 0;
+      if (nN) atomicAdd((unsigned long long *)&s.ctr->cache_lw, (unsigned long long)nN);
+    }
     __syncwarp();
   }
 }
@@ -1633,6 +1637,7 @@ void fill_query_args(hac_ctx *h, QueryArgs &qa, int round, int K, int nterm) {
   qa.cval = s.cval;
   qa.cerr = s.cerr;
   qa.cpart = s.cpart;
+  qa.cused = s.cused;
   qa.gen = s.gen;
   qa.ins_i = s.ins_i;
   qa.ins_j = s.ins_j;
@@ -1682,9 +1687,10 @@ bool use_brute(const hac_ctx *h) {
 // Searches for groups of terminals (hac_gsearch.cu): the closed-form linkages in
 // d <= 8, one instance, unless the ablation wants every cluster scanned or the
 // FP32 squares could flush or overflow.
-bool use_gsearch(const hac_ctx *h) {
+bool use_gsearch(const hac_ctx *h, int K) {
   const State &s = h->s;
-  return closed_form(s.linkage) && s.max_inst == 1 && !s.noprune && s.d <= 8 &&
+  // (a pair of single points is the one case of the others that needs no more)
+  return (closed_form(s.linkage) || K == h->n) && s.max_inst == 1 && !s.noprune && s.d <= 8 &&
          s.coord_scale >= (float)FIN_SCALE_LO && s.coord_scale < (float)FIN_SCALE_HI;
 }
 
@@ -1760,13 +1766,14 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
   } else if (brute) {
     CK(launch_brute(qa, s.dp, device_sms(), st));
     h->launches += 3;
-  } else if (use_gsearch(h)) {
-    CK(cudaMemsetAsync(&s.ctr->npend, 0, sizeof(int32_t), st));
-    qa.pend_out = s.blist;
-    CK(launch_gsearch(qa, st));
-    QueryArgs rest = qa;  // the near ties it left undecided
+  } else if (!qa.lcnt && use_gsearch(h, K)) {
+    CK(cudaMemsetAsync(&s.ctr->nrq, 0, sizeof(int32_t), st));
+    QueryArgs rest = qa;  // the near ties it leaves undecided
     rest.term = s.blist;
-    rest.nterm_dev = &s.ctr->npend;
+    rest.nterm_dev = &s.ctr->nrq;
+    qa.pend_out = s.blist;
+    CK(launch_gsearch(qa, query_prec(s), st));
+    qa.pend_out = rest.pend_out;
     CK(launch_query(rest, s.dp, query_prec(s), st));
     h->launches += 1;
   } else {
@@ -2180,7 +2187,8 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
     if (!s.ins_i) {  // queue of evaluated pairs to insert (sized once per handle)
       const int64_t cap = std::max<int64_t>(4 * h->n, 1 << 16);
       if ((rc0 = dalloc(h, &s.ins_i, cap)) || (rc0 = dalloc(h, &s.ins_j, cap)) ||
-          (rc0 = dalloc(h, &s.ins_v, cap)) || (rc0 = dalloc(h, &s.ins_e, cap)))
+          (rc0 = dalloc(h, &s.ins_v, cap)) || (rc0 = dalloc(h, &s.ins_e, cap)) ||
+          (rc0 = dalloc(h, &s.cused, h->n)))
         return rc0;
       s.ins_cap = (int)cap;
     }
@@ -2215,8 +2223,10 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
     h->cache_alloc_slots = slots;
   }
   s.cache_slots = slots;
-  if (slots > 0)
+  if (slots > 0) {
     CK(cudaMemsetAsync(s.ckey, 0xff, (size_t)h->n * slots * sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(s.cused, 0, h->n, st));
+  }
   h->st = hac_stats_t{};
   h->st.device_bytes = h->bytes;
   const auto t0 = std::chrono::steady_clock::now();

@@ -1,4 +1,6 @@
-// Nearest-neighbour search of Ward and avg-2 for groups of terminals at once.
+// Nearest-neighbour search of Ward and avg-2 for groups of terminals at once, and
+// of complete and average linkage in the first round, whose pairs of single
+// points are plain distances.
 //
 // The search of hac_query.cuh gives every terminal a warp, whose lanes share
 // the tree nodes and bucket records; at 10^6 points in 5-D a search is some 25
@@ -114,6 +116,7 @@ struct GTerm {
   // squared distance that passes beside a record (or node) with 1 / size gb
   // (largest under the node), Ward; avg-2: minus the variances
   __device__ float limit(float gb) const {
+    // (single points of complete and average linkage: variances of 0)
     return LK == LK_WARD ? 0.5f * tq * (g + gb) : tq - g - gb;
   }
 };
@@ -127,7 +130,8 @@ struct GCount {
 // terminals reach so far that they are to be searched alone.
 template <int LK, int D, int DP, int G>
 __device__ __forceinline__ unsigned g_search(const QueryArgs &a, const int *s_ti, uint32_t *sn,
-                                             float *sd, int lane, int ci, bool act, GCount &n) {
+                                             float *sd, int lane, int ci, bool act, bool f32,
+                                             GCount &n) {
   constexpr int S = 32 / G;  // lanes per terminal
   constexpr int B = G == 1 ? 1 : D <= 3 ? 4 : 2;
   const int slice = lane / G;
@@ -318,22 +322,35 @@ __device__ __forceinline__ unsigned g_search(const QueryArgs &a, const int *s_ti
   const bool one = T.p1 >= 0 && T.L1 * (1.f - rho2) <= lim && T.L2 * (1.f - rho2) > lim;
   if (act && slice == 0) {
     if (one && !alone) {
-      const int cb = a.order[T.p1], nb = a.qsz[T.p1];
-      const int na = a.qsz[T.pos];
-      double s = 0.0;
+      const int cb = a.order[T.p1];
+      double key;
+      if (LK == LK_COMPLETE || LK == LK_AVERAGE) {
+        // as the search of hac_query.cuh: in the FP32 mode the upper bound of the
+        // FP32 distance where that is within 4e-6, else the FP64 distance
+        const float d1 = f32 ? eval32_lane<LK, DP>(a.p32, a.qseg[T.pos], 1, a.qseg[T.p1], 1) : 0.f;
+        const float rho = ((float)a.d + 16.f) * U32 + (LK == LK_AVERAGE ? 32.f * U32 : 0.f);
+        const float e1 = a.delta_pts;
+        if (f32 && e1 + rho * d1 <= 4e-6f * d1)
+          key = (double)((d1 + e1) * (1.f + rho));
+        else
+          key = eval64_lane<LK, DP>(a.p64, a.qseg[T.pos], 1, a.qseg[T.p1], 1);
+      } else {
+        const int na = a.qsz[T.pos], nb = a.qsz[T.p1];
+        double s = 0.0;
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        if (k < a.d) {
-          const double u = a.q64[(size_t)T.pos * DP + k] - a.q64[(size_t)T.p1 * DP + k];
-          s += u * u;
+        for (int k = 0; k < D; ++k) {
+          if (k < a.d) {
+            const double u = a.q64[(size_t)T.pos * DP + k] - a.q64[(size_t)T.p1 * DP + k];
+            s += u * u;
+          }
         }
+        key = LK == LK_AVG2 ? s + a.sse[ci] / (double)na + a.sse[cb] / (double)nb
+                            : (2.0 * (double)na * (double)nb) / (double)(na + nb) * s;
       }
-      a.Ekey[ci] = LK == LK_AVG2
-                       ? s + a.sse[ci] / (double)na + a.sse[cb] / (double)nb
-                       : (2.0 * (double)na * (double)nb) / (double)(na + nb) * s;
+      a.Ekey[ci] = key;
       a.Ecid[ci] = cb;
     } else if (!alone) {
-      a.pend_out[atomicAdd(&a.ctr->npend, 1)] = ci;
+      a.pend_out[atomicAdd(&a.ctr->nrq, 1)] = ci;
     }
   }
   __syncwarp();
@@ -341,7 +358,7 @@ __device__ __forceinline__ unsigned g_search(const QueryArgs &a, const int *s_ti
 }
 
 template <int LK, int D, int DP, int G>
-__global__ void __launch_bounds__(GW * 32) k_gsearch(QueryArgs a) {
+__global__ void __launch_bounds__(GW * 32) k_gsearch(QueryArgs a, bool f32) {
   __shared__ uint32_t s_node[GW][GSTK];
   __shared__ float s_need[GW][GSTK];
   __shared__ int s_ti[TI_SIZE];
@@ -359,10 +376,10 @@ __global__ void __launch_bounds__(GW * 32) k_gsearch(QueryArgs a) {
   const int ci = a.term[min(t, a.nterm - 1)];
   GCount n{0, 0, 0};
   unsigned far = g_search<LK, D, DP, G>(a, s_ti, s_node[wib], s_need[wib], lane, ci,
-                                        t < a.nterm, n);
+                                        t < a.nterm, f32, n);
   for (; far; far &= far - 1)
     g_search<LK, D, DP, 1>(a, s_ti, s_node[wib], s_need[wib], lane,
-                           __shfl_sync(0xffffffffu, ci, __ffs(far) - 1), true, n);
+                           __shfl_sync(0xffffffffu, ci, __ffs(far) - 1), true, f32, n);
   n.offers = __reduce_add_sync(0xffffffffu, n.offers);
   if (lane == 0) {
     atomicAdd(&a.ctr->cluster_pairs, (unsigned long long)n.offers);
@@ -372,7 +389,7 @@ __global__ void __launch_bounds__(GW * 32) k_gsearch(QueryArgs a) {
 }
 
 template <int LK, int D>
-cudaError_t launch_g(const QueryArgs &a, cudaStream_t s) {
+cudaError_t launch_g(const QueryArgs &a, bool f32, cudaStream_t s) {
   constexpr int DP = D <= 2 ? 2 : D <= 4 ? 4 : 8;
   constexpr int W = D <= 2 ? GS_W2 : GS_W;
   const bool wide = a.nterm >= GS_WIDE;
@@ -380,32 +397,39 @@ cudaError_t launch_g(const QueryArgs &a, cudaStream_t s) {
   const int groups = (a.nterm + G - 1) / G;
   const int blocks = (groups + GW - 1) / GW;
   if (wide)
-    k_gsearch<LK, D, DP, W><<<blocks, GW * 32, 0, s>>>(a);
+    k_gsearch<LK, D, DP, W><<<blocks, GW * 32, 0, s>>>(a, f32);
   else
-    k_gsearch<LK, D, DP, GS_N><<<blocks, GW * 32, 0, s>>>(a);
+    k_gsearch<LK, D, DP, GS_N><<<blocks, GW * 32, 0, s>>>(a, f32);
   return cudaGetLastError();
 }
 
 template <int LK>
-cudaError_t launch_glk(const QueryArgs &a, cudaStream_t s) {
+cudaError_t launch_glk(const QueryArgs &a, bool f32, cudaStream_t s) {
   switch (a.d) {
-    case 1: return launch_g<LK, 1>(a, s);
-    case 2: return launch_g<LK, 2>(a, s);
-    case 3: return launch_g<LK, 3>(a, s);
-    case 4: return launch_g<LK, 4>(a, s);
-    case 5: return launch_g<LK, 5>(a, s);
-    case 6: return launch_g<LK, 6>(a, s);
-    case 7: return launch_g<LK, 7>(a, s);
-    case 8: return launch_g<LK, 8>(a, s);
+    case 1: return launch_g<LK, 1>(a, f32, s);
+    case 2: return launch_g<LK, 2>(a, f32, s);
+    case 3: return launch_g<LK, 3>(a, f32, s);
+    case 4: return launch_g<LK, 4>(a, f32, s);
+    case 5: return launch_g<LK, 5>(a, f32, s);
+    case 6: return launch_g<LK, 6>(a, f32, s);
+    case 7: return launch_g<LK, 7>(a, f32, s);
+    case 8: return launch_g<LK, 8>(a, f32, s);
   }
   return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t launch_gsearch(const QueryArgs &a, cudaStream_t s) {
+cudaError_t launch_gsearch(const QueryArgs &a, int prec, cudaStream_t s) {
   if (a.nterm <= 0) return cudaSuccess;
-  return a.linkage == LK_WARD ? launch_glk<LK_WARD>(a, s) : launch_glk<LK_AVG2>(a, s);
+  const bool f32 = prec != 0;
+  switch (a.linkage) {
+    case LK_COMPLETE: return launch_glk<LK_COMPLETE>(a, f32, s);
+    case LK_AVERAGE: return launch_glk<LK_AVERAGE>(a, f32, s);
+    case LK_WARD: return launch_glk<LK_WARD>(a, f32, s);
+    case LK_AVG2: return launch_glk<LK_AVG2>(a, f32, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace hacg

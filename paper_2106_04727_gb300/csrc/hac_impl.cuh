@@ -66,7 +66,10 @@ __device__ inline void cache_insert(const State &s, int owner, int nbr, int nbr_
         return;
       }
       if (!slot_free(s, cur)) break;
-      if (slot_put(s, base + t, cur, want, v, e)) return;
+      if (slot_put(s, base + t, cur, want, v, e)) {
+        s.cused[owner] = 1;
+        return;
+      }
     }
   }
 }

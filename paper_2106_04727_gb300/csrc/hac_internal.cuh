@@ -97,6 +97,8 @@ struct State {
   // D(owner, neighbour); c > 0 = it is D(first c points of the owner,
   // neighbour); c < 0 = D(last -c points of the owner, neighbour)
   int32_t *cpart;
+  uint8_t *cused;       // 0 while nothing has been put into the table of a cid: its
+                        // slots need no look (small clusters never have entries)
   int ins_cap;          // queue of evaluated pairs to insert after the search
   int32_t *ins_i, *ins_j;
   double *ins_v;
@@ -241,6 +243,7 @@ struct QueryArgs {
   const double *cval;
   const float *cerr;
   const int32_t *cpart;
+  const uint8_t *cused;
   const int32_t *gen;
   int32_t *ins_i, *ins_j;
   double *ins_v;
@@ -353,9 +356,10 @@ constexpr int TI_SIZE = MAXLEV + 3;
 // launches the nearest-neighbour query of every terminal (hac_query.cu)
 cudaError_t launch_query(const QueryArgs &a, int dp, int prec, cudaStream_t s);
 // the same search for Ward / avg-2 with d <= 8, one instance, for groups of
-// terminals (hac_gsearch.cu): leaves undecided terminals in pend_out and
-// ctr->npend (zeroed first) to launch_query (nterm_dev = &ctr->npend)
-cudaError_t launch_gsearch(const QueryArgs &a, cudaStream_t s);
+// terminals (hac_gsearch.cu); complete and average while every cluster is a
+// single point: leaves undecided terminals in pend_out and ctr->nrq (zeroed
+// first) to launch_query (nterm_dev = &ctr->nrq)
+cudaError_t launch_gsearch(const QueryArgs &a, int prec, cudaStream_t s);
 #ifndef HAC_GS_WIDE
 #define HAC_GS_WIDE 40000
 #endif

@@ -485,6 +485,7 @@ struct Searcher {
   // (warp-cooperative; valid only while the neighbour's generation matches)
   // (`part` receives the entry's partial tag, 0 for a full value)
   __device__ bool cache_find(int owner, int nbr, double &v, float &e, int &part) const {
+    if (!a.cused[owner]) return false;
     const int S = a.cache_slots;
     const unsigned long long want = ckey_of(nbr, a.gen[nbr]);
     for (int base = 0; base < S; base += 32) {

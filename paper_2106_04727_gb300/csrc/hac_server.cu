@@ -173,6 +173,7 @@ __global__ void k_admit_layout(State s, const T *stage, int m, const AdmitInst *
     s.qseg[op] = (int32_t)pp;
     s.qinst[op] = a.seq;
     for (int q = 0; q < s.cache_slots; ++q) s.ckey[(size_t)c * s.cache_slots + q] = CKEY_EMPTY;
+    if (s.cache_slots > 0) s.cused[c] = 0;
   }
 }
 
@@ -317,6 +318,7 @@ int engine_init(Engine &e, hac_linkage lk, int d, hac_dtype dt, int64_t cap, con
     m.add(&s.cval, cells);
     m.add(&s.cerr, cells);
     m.add(&s.cpart, cells);
+    m.add(&s.cused, cap);
     m.add(&s.breq_base, bcap);
     m.add(&s.breq_cov, bcap);
     m.add(&s.breq_berr, bcap);

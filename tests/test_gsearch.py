@@ -54,3 +54,24 @@ def test_hard_inputs(lk, kind):
         X = np.concatenate([1e-3 * inputs.gaussian_mixture(4600, 4, 6, seed=3),
                             np.full((1, 4), 1e5, np.float32), np.full((1, 4), -3e4, np.float32)])
     _check(hac.cluster(X, lk), hac.cluster(X, lk, no_prune=True), rtol=1e-12)
+
+
+@pytest.mark.parametrize("prec", [hac.PREC_F64, hac.PREC_F32_RECHECK], ids=["f64", "f32recheck"])
+@pytest.mark.parametrize("lk", ["complete", "average"])
+@pytest.mark.parametrize("d", list(range(1, 9)))
+def test_single_points(lk, d, prec, monkeypatch):
+    """The first round of complete and average linkage (no dense matrix)."""
+    monkeypatch.setenv("HAC_DENSE_K", "0")
+    X = inputs.gaussian_mixture(2500 + 7 * d, d, 9, seed=70 + d,
+                                dtype=np.float64 if d % 2 else np.float32)
+    got = hac.cluster(X, lk, precision=prec, cache_slots=16)
+    _check(got, oracle.rounds(X.astype(np.float64), lk),
+           rtol=1e-9 if prec == hac.PREC_F64 else 1e-5)
+
+
+@pytest.mark.parametrize("lk", ["complete", "average"])
+def test_single_points_ties(lk, monkeypatch):
+    monkeypatch.setenv("HAC_DENSE_K", "0")
+    X = inputs.lattice(3000, 2, seed=12, levels=30)
+    got = hac.cluster(X, lk, precision=hac.PREC_F32_RECHECK, cache_slots=16)
+    _check(got, hac.cluster(X, lk, cache_slots=16), rtol=1e-5)
