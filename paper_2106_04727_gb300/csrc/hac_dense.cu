@@ -1825,8 +1825,10 @@ int dense_alloc(hac_ctx *h, int64_t cap) {
 //   d = 2, 100,000 points: 10.4 at 4,096, 11.2 at 8,192; 10^6: 170 / 168
 //   d = 5, 20,001 points: 11.0 at 4,096, 11.8 at 8,192, 20.4 at 16,384;
 //     200,000: 64.8 at 4,096, 49.7 at 8,192; 10^6: 463 / 440 / 426 at 16,384
-//   d = 10, 20,001 points: 19.5 from the start, 28.8 at 8,192; 16-D lattice,
-//     10^6 points: 11.5 s at 32,768, 8.3 s at 65,536
+//   d = 10, 20,001 points: 19.5 from the start, 28.8 at 8,192; 30,001: 37.9
+//     from the start, 42.7 at 16,384; 100,000: 191 at 16,384, 189 at 20,000,
+//     190 at 32,768 (and 16 GB less to allocate); 16-D lattice, 10^6 points:
+//     11.5 s at 32,768, 8.3 s at 65,536
 // complete (from the start or not at all): FP32 d = 2, 20,001 points 8.6
 // against 13.1 on the range query, 30,001: 15.5 / 14.2; d = 5, 30,001: 19.6 /
 // 22.0, 32,768: 23.8 / 22.9; FP64, whose point pairs cost 60 times as much,
@@ -1838,7 +1840,7 @@ int64_t dense_default(int64_t n, int d, int linkage, int prec) {
   if (linkage == LK_COMPLETE)
     k = prec == HAC_PREC_F64 || d > 8 ? 32768 : d <= 3 ? 24576 : 30000;
   else if (d > 8)
-    k = 65536;
+    k = n <= 32768 ? 32768 : std::min<int64_t>(65536, std::max<int64_t>(20000, n / 16));
   else if (n <= 8192)
     k = 8192;
   else if (d <= 3)
