@@ -137,7 +137,8 @@ typedef struct {
   int64_t dense_point_pairs; /* point pairs of the all-pairs sweep that filled it (also
                                 in point_pairs) */
   int64_t dense_rechecks;    /* FP32 mode: matrix entries re-scored in FP64 */
-  double ms_dense;           /* device time of filling the matrix */
+  double ms_dense;           /* device time of the sweep, or of the matrix's fill from
+                                single points */
 } hac_stats_t;
 
 /* Default options (FP64, no cache, no limits, own stream).  No counterpart in

@@ -1732,14 +1732,20 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
   const bool defer = !dense && qa.defer != 0;
   if (defer)
     CK(cudaMemsetAsync(s.side_key, 0xff, (size_t)s.side_cap * sizeof(unsigned long long), st));
-  const bool brute = !dense && use_brute(h);
+  bool brute = !dense && use_brute(h);
+  if (brute && !s.glist) {  // sized once per handle
+    SlabAlloc m;
+    m.add(&s.gu, h->n);
+    m.add(&s.gcnt, h->n);
+    m.add(&s.glist, (size_t)h->n * GRAM_LIST);
+    if (m.commit(h)) {  // no room: the instance stays on the tree search
+      h->brute_env = 0;
+      brute = false;
+    }
+  }
   if (brute) {
     CK(cudaMemsetAsync(&s.ctr->npend, 0, sizeof(int32_t), st));
     qa.pend_out = s.blist;
-    if (!s.glist &&  // sized once per handle
-        ((rc = dalloc(h, &s.gu, h->n)) || (rc = dalloc(h, &s.gcnt, h->n)) ||
-         (rc = dalloc(h, &s.glist, (size_t)h->n * GRAM_LIST))))
-      return rc;
     qa.gu = s.gu;
     qa.gcnt = s.gcnt;
     qa.glist = s.glist;

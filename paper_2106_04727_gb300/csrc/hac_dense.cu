@@ -1895,10 +1895,10 @@ int dense_maybe_enter(hac_ctx *h, cudaStream_t st, int K, RoundCtl &ctl) {
   const bool f32 = s.prec == HAC_PREC_F32_RECHECK;
   const bool single = (int64_t)K == h->lay_n;
   double *b0 = h->dense_buf, *b1 = b0 + h->dense_stride, *b2 = b1 + h->dense_stride;
-  if (ctl.eb0) cudaEventRecord(ctl.eb0, st);
   k_dense_init<<<grid_for(K, TPB), TPB, 0, st>>>(
       s, s.order[h->ocur], K, single ? (unsigned long long)K * (K - 1) / 2 : 0ull);
   if (single) {
+    if (ctl.eb0) cudaEventRecord(ctl.eb0, st);
     const float inv_scl = std::ldexp(1.0f, -k);
     if (s.linkage == LK_COMPLETE) {
       s.dmat = b0;
@@ -1917,6 +1917,7 @@ int dense_maybe_enter(hac_ctx *h, cudaStream_t st, int K, RoundCtl &ctl) {
         launch_single<LK_AVERAGE, 0>(h, st, K, scl, es, inv_scl);
     }
     CK(cudaGetLastError());
+    if (ctl.eb1) cudaEventRecord(ctl.eb1, st);
   } else {
     const size_t cells = (size_t)K * (K - 1) / 2;
     CK(cudaMemsetAsync(b0, 0, cells * LIMBS * sizeof(unsigned long long), st));
@@ -1932,8 +1933,10 @@ int dense_maybe_enter(hac_ctx *h, cudaStream_t st, int K, RoundCtl &ctl) {
     a.es = es;
     a.sum = (unsigned long long *)b0;
     a.ctr = s.ctr;
+    if (ctl.eb0) cudaEventRecord(ctl.eb0, st);
     int rc = sweep(h, st, a);
     if (rc) return rc;
+    if (ctl.eb1) cudaEventRecord(ctl.eb1, st);
     k_dense_pack<<<grid_for((int64_t)cells, TPB), TPB, 0, st>>>(
         (const unsigned long long *)b0, (unsigned long long *)b2, cells, f32);
     s.dsum = (unsigned long long *)b2;
@@ -1944,7 +1947,6 @@ int dense_maybe_enter(hac_ctx *h, cudaStream_t st, int K, RoundCtl &ctl) {
     h->launches += 2;
     ctl.dense_launches += 2;
   }
-  if (ctl.eb1) cudaEventRecord(ctl.eb1, st);
   if (ctl.eb0) {
     CK(cudaEventSynchronize(ctl.eb1));
     float ms = 0.f;
