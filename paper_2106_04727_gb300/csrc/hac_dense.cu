@@ -402,12 +402,16 @@ __device__ __forceinline__ void flush(const SweepArgs &a, const U128 (&acc)[PPT]
 // Two of a thread's rows share each f32x2 word (one coordinate of each) and
 // every staged column is duplicated into both halves, so one packed subtract
 // and one packed multiply-add advance two point pairs by one coordinate.  Per
-// row and column segment: FP32 partial sums of at most 32 terms, each
-// converted to fixed point exactly and added as integers (no FP64 work).
+// row and column segment: FP32 partial sums of at most 32 terms (two rows' sums
+// per packed word), each converted to fixed point exactly and added as integers
+// (no FP64 work).  Columns are staged padded to whole 16-byte words: 3 instead of
+// 5 loads and 2 instead of 4 additions per column at d = 5 took the sweep of 10^6
+// points from 220 to 206 ms (17 flops per pair: 41 TFLOP/s of the 80 measured).
 template <int D, int DP, int PPT>
 __global__ void __launch_bounds__(DS_TPB, HAC_DS_MINB) k_dense_sweep32(SweepArgs a) {
   constexpr int TI = DS_TPB * PPT, NP = PPT / 2;
-  __shared__ unsigned long long sy[DS_CH * D];
+  constexpr int DE = (D + 1) & ~1;  // staged columns are read 16 bytes at a time
+  __shared__ __align__(16) unsigned long long sy[DS_CH * DE];
   __shared__ int skey[DS_CH];
   __shared__ int sstart[DS_CH + 1];
   __shared__ int wtot[DS_TPB / 32];
@@ -438,7 +442,7 @@ __global__ void __launch_bounds__(DS_TPB, HAC_DS_MINB) k_dense_sweep32(SweepArgs
     for (int i = threadIdx.x; i < cnt * D; i += DS_TPB) {
       const int c = i / D, k = i - c * D;
       const float y = a.p32[(size_t)(c0 + c) * DP + k] * a.scl;
-      sy[i] = f2_pack(y, y);
+      sy[c * DE + k] = f2_pack(y, y);
     }
     if (threadIdx.x < DS_CH)
       skey[threadIdx.x] = threadIdx.x < cnt ? a.pos[a.plab[c0 + threadIdx.x]] : -1;
@@ -453,14 +457,18 @@ __global__ void __launch_bounds__(DS_TPB, HAC_DS_MINB) k_dense_sweep32(SweepArgs
       for (int r = 0; r < PPT; ++r) acc[r] = U128{0ull, 0ull};
       for (int c1 = cb; c1 < ce; c1 += 32) {
         const int c2 = min(c1 + 32, ce);
-        float part[PPT];
+        unsigned long long part[NP];  // two rows' sums per word
 #pragma unroll
-        for (int r = 0; r < PPT; ++r) part[r] = 0.f;
+        for (int h = 0; h < NP; ++h) part[h] = 0ull;
 #pragma unroll 2
         for (int c = c1; c < c2; ++c) {
-          unsigned long long y[D];
+          unsigned long long y[DE];
 #pragma unroll
-          for (int k = 0; k < D; ++k) y[k] = sy[c * D + k];
+          for (int k = 0; k < DE; k += 2) {
+            const ulonglong2 w = *(const ulonglong2 *)&sy[c * DE + k];
+            y[k] = w.x;
+            y[k + 1] = w.y;
+          }
 #pragma unroll
           for (int h = 0; h < NP; ++h) {
             unsigned long long t = f2_sub(x[h][0], y[0]);
@@ -472,12 +480,16 @@ __global__ void __launch_bounds__(DS_TPB, HAC_DS_MINB) k_dense_sweep32(SweepArgs
             }
             float s0, s1;
             f2_unpack(d2, s0, s1);
-            part[2 * h] += sqrt_approx_ftz(s0);
-            part[2 * h + 1] += sqrt_approx_ftz(s1);
+            part[h] = f2_add(part[h], f2_pack(sqrt_approx_ftz(s0), sqrt_approx_ftz(s1)));
           }
         }
 #pragma unroll
-        for (int r = 0; r < PPT; ++r) u128_add(acc[r], fx_of_f(part[r], a.es));
+        for (int h = 0; h < NP; ++h) {
+          float p0, p1;
+          f2_unpack(part[h], p0, p1);
+          u128_add(acc[2 * h], fx_of_f(p0, a.es));
+          u128_add(acc[2 * h + 1], fx_of_f(p1, a.es));
+        }
       }
       int below = 0;
 #pragma unroll
