@@ -583,13 +583,24 @@ constexpr int FT_Y = 8;
 
 __device__ __forceinline__ bool fin_tile(int K, long long &ti, long long &tj) {
   // consecutive blocks take consecutive tiles of one tile row, so the rows of
-  // sums and means in flight together are long
+  // sums and means in flight together are long.  One warp works the tile out,
+  // not all eight: the FP64 square root in tile_of helped to keep the FP64 pipe
+  // 63 % busy in the fill (rebuilds of an average run of 20,001 10-D points 8.2
+  // ms, 7.3 this way; its fill 2.9, 2.7).
+  __shared__ long long s_tile[2];
   const int nt = (K + 31) / 32;
-  long long bi, bj;
-  tile_of(blockIdx.x + (long long)gridDim.x * blockIdx.y, bi, bj);
-  ti = nt - 1 - bj;
-  tj = nt - 1 - bi;
-  return bi < nt && bj < nt;
+  if (threadIdx.y == 0) {
+    long long bi, bj;
+    tile_of(blockIdx.x + (long long)gridDim.x * blockIdx.y, bi, bj);
+    if (threadIdx.x == 0) {
+      s_tile[0] = nt - 1 - bj;
+      s_tile[1] = nt - 1 - bi;
+    }
+  }
+  __syncthreads();
+  ti = s_tile[0];
+  tj = s_tile[1];
+  return ti >= 0 && tj >= 0;
 }
 
 // upper tile in Mv (row k, column tx) -> both triangles of the mean matrix
@@ -659,7 +670,7 @@ __device__ __noinline__ double dist64(const double *x, const double *y, int d) {
 // root; FP64: the same fma chain).  Bound by the 24-32 B written per pair, or
 // in FP64 by the square roots; the segmented sweep, which flushes every column
 // of every row through atomics when each point is a cluster of its own, took
-// 11 ms with its last pass at 20,001 points in 10-D, this 2.9.
+// 11 ms with its last pass at 20,001 points in 10-D, this 2.7.
 template <int LK, int DP, int F32>
 __global__ void __launch_bounds__(32 * FT_Y) k_dense_single(State s, const float *p32,
                                                              const double *p64, int K, float scl,
@@ -1071,7 +1082,7 @@ __global__ void k_drq_fin(State s, int m) {
 // and each new one written once, all in row segments (average: 8 K^2 B of
 // sums read, 8 K'^2 B of sums and 8 K'^2 B of means written), and later scans
 // read no dead columns.  Patching in place (scattered column writes and
-// packed-column reads) took 18.9 ms at 20,001 points in 10-D, this 8.2 with
+// packed-column reads) took 18.9 ms at 20,001 points in 10-D, this 7.3 with
 // the compactions of the lists; the row scans fell from 14.6 to 7.5 ms.
 // Average linkage: the sum of A u B with C is the sum of A's and B's (exact),
 // the mean follows from the new sizes.  Complete: the larger entry.
