@@ -10,8 +10,9 @@
 // buckets, so here a warp searches for G of them together: one lane per
 // terminal (32 / G lanes share a terminal's records when G < 32).  Records are
 // read by uniform loads, tested against every lane's own threshold in FP32, and
-// a bucket is scanned if any lane needs it; inner nodes are pruned with the
-// group's box, its smallest size and its largest threshold.  FP64 keys are
+// a node is opened, or a bucket scanned, if any lane itself reaches its box;
+// before that, all children of a node at once are pruned with the group's box,
+// its smallest size and its largest threshold.  FP64 keys are
 // computed once per terminal at the end, all lanes at a time.
 //
 // Bounds.  Every test is on FP32 squared distances of the same FP32 records, and
@@ -27,13 +28,20 @@
 // scans more records per terminal and fewer instructions per record.  Measured,
 // Ward whole runs of 10^6 points (ms, group size from GS_WIDE terminals on):
 // 2-D 17.0 / 17.2 / 17.2 (8 / 16 / 32), 5-D 45.6 / 47.4 / 54.3, 8-D 96.4 / 94.3 /
-// 107.9; the warp-per-terminal search: 27.6, 59.5, 170.  10^7 2-D points have
+// 107.9; the warp-per-terminal search: 27.6, 59.5, 170.  (With the group's bounds
+// alone for inner nodes.  Each lane's own test of the popped node, for groups that
+// span a gap of the spatial order: 5-D 42.7 -> 33.0 with 8.)  10^7 2-D points have
 // enough terminals for the widest: first round 9.8 ms with 8, 4.2 with 32 (43
 // before).  Below that few groups
 // leave warps idle: 60,000 points in 5-D 7.5 with 4, 8.2 with 8 (9.8 before).
 // A terminal that reaches much farther than its group (a large cluster among
 // singletons: a node's bound knows only its smallest size) is searched by the
 // whole warp alone; leaving it in the group cost 11 of 57 ms in 5-D.
+//
+// A node's nearest child is visited first.  In index order a terminal alone in its
+// bucket beside a dense line of points came in from the far end of the tree: whole
+// Ward run of 10^7 clipped 2-D Gaussians 396 ms, 62 nearest first (202 with the
+// warp-per-terminal search); 10^7 2-D spreaders 77 and 54.
 #include "hac_query.cuh"
 
 namespace hacg {
@@ -266,8 +274,15 @@ __device__ __forceinline__ unsigned g_search(const QueryArgs &a, const int *s_ti
       if (lane == 0) atomicOr(&a.ctr->err, ERR_STACK);
       return top;
     }
+    // The nearest child goes on top: a terminal alone in its bucket starts without
+    // a bound, and has one after the first bucket of this descent (in index order
+    // it would come in from the far end of the tree, bucket by bucket).
+    const unsigned kn = ok ? __float_as_uint(need) : 0xffffffffu;  // need >= 0
+    const unsigned best = __reduce_min_sync(0xffffffffu, kn);
+    const int fl = __ffs(__ballot_sync(0xffffffffu, ok && kn == best)) - 1;
     if (ok) {
-      const int at = top + __popc(m & ((1u << lane) - 1u));
+      const int at = top + (lane == fl ? __popc(m) - 1
+                                       : __popc(m & ((1u << lane) - 1u)) - (fl < lane));
       sn[at] = ((uint32_t)L << 28) | (uint32_t)child;
       sd[at] = need;
     }
@@ -283,24 +298,28 @@ __device__ __forceinline__ unsigned g_search(const QueryArgs &a, const int *s_ti
     __syncwarp();
     if (need > TQ) continue;
     const int L = (int)(e >> 28), j = (int)(e & ((1u << 28) - 1));
-    if (L > 0) {
-      const int c0 = a.nch[a.chb[L] + j];
-      top = push(top, L - 1, c0, a.nch[a.chb[L] + j + 1] - c0);
-      continue;
-    }
-    if (__any_sync(0xffffffffu, own == j)) continue;  // scanned first
-    // does any terminal itself reach the bucket's box?
+    if (L == 0 && __any_sync(0xffffffffu, own == j)) continue;  // scanned first
+    // does any terminal itself reach the node's box?  (The group's box may span
+    // a gap of the spatial order, with a dense region inside it that no terminal
+    // reaches.)
+    const int node = a.lvl_base[L] + j;
     float lo[D], hi[D];
-    g_load<D, DP>(a.nclo + (size_t)j * DP, lo);
-    g_load<D, DP>(a.nchi + (size_t)j * DP, hi);
+    g_load<D, DP>(a.nclo + (size_t)node * DP, lo);
+    g_load<D, DP>(a.nchi + (size_t)node * DP, hi);
     float dc2 = 0.f;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
       const float u = fmaxf(fmaxf(lo[k] - T.x[k], T.x[k] - hi[k]), 0.f);
       dc2 = fmaf(u, u, dc2);
     }
-    const float gb = LK == LK_WARD ? g_rcp((float)a.nnmin[j]) * (1.f + 1e-6f) : 0.f;
-    if (__any_sync(0xffffffffu, !alone && dc2 <= T.limit(gb))) scan(j);
+    const float gb = LK == LK_WARD ? g_rcp((float)a.nnmin[node]) * (1.f + 1e-6f) : 0.f;
+    if (!__any_sync(0xffffffffu, !alone && dc2 <= T.limit(gb))) continue;
+    if (L > 0) {
+      const int c0 = a.nch[a.chb[L] + j];
+      top = push(top, L - 1, c0, a.nch[a.chb[L] + j + 1] - c0);
+    } else {
+      scan(j);
+    }
   }
   // the lanes of one terminal together
   if (S > 1) {

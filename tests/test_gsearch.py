@@ -40,7 +40,7 @@ def test_wide_groups(lk, name, n):
 
 
 @pytest.mark.parametrize("lk", LKS)
-@pytest.mark.parametrize("kind", ["lattice", "duplicates", "line", "outliers"])
+@pytest.mark.parametrize("kind", ["lattice", "duplicates", "line", "outliers", "clipped", "gap"])
 def test_hard_inputs(lk, kind):
     """The same tree as with every cluster scanned in FP64 (no pruning, no
     grouping)."""
@@ -50,6 +50,12 @@ def test_hard_inputs(lk, kind):
         X = np.repeat(inputs.gaussian_mixture(450, 3, 5, seed=7), 10, axis=0)
     elif kind == "line":
         X = np.arange(4500, dtype=np.float32)[:, None] * np.float32(0.5)
+    elif kind == "clipped":  # points alone in their bucket beside a dense line
+        X = inputs.uniform_cube(6000, 2, seed=21, dtype=np.float32)
+        X[:3000, 1] = 1.0
+    elif kind == "gap":  # groups whose box holds a dense region none of them reaches
+        X = inputs.uniform_cube(6000, 2, seed=22, dtype=np.float32)
+        X[:4000] = np.float32(0.498) + X[:4000] * np.float32(0.004)
     else:
         X = np.concatenate([1e-3 * inputs.gaussian_mixture(4600, 4, 6, seed=3),
                             np.full((1, 4), 1e5, np.float32), np.full((1, 4), -3e4, np.float32)])
