@@ -151,7 +151,9 @@ void hac_default_opts(hac_opts *opts);
  * `dt` (float or double), read during the call and not retained.  Allocates
  * all device memory the instance needs; the points are copied to the device.
  * HAC_EINVAL: points/out NULL, n < 1, d < 1 or d > 16, unknown dt/lk, or a
- * non-finite coordinate.  HAC_ENOMEM: device allocation failed. */
+ * non-finite coordinate.  HAC_ENOMEM: device allocation failed.  Coordinates of
+ * any finite magnitude are taken: an input far from unit scale is clustered times
+ * a power of two, and its heights are multiplied back. */
 int hac_create(const void *points, int64_t n, int d, hac_dtype dt, hac_linkage lk, hac_t *out);
 
 /* (Paper: as hac_create, Algorithm 1's input.)  As hac_create, but

@@ -208,6 +208,7 @@ __global__ void k_bbox(const T *X, int64_t n, int d, unsigned long long *mn,
 
 struct MortonParams {
   double lo[MAXD], inv[MAXD];
+  double mul;  // power of two every coordinate is multiplied by
   int bits;
 };
 
@@ -247,7 +248,7 @@ __global__ void k_layout_cid(State s, const T *X, MortonParams ctr_) {
        i += (int64_t)gridDim.x * blockDim.x) {
     double sq = 0.0;
     for (int k = 0; k < dp; ++k) {
-      const double x = k < d ? (double)X[i * d + k] - ctr_.lo[k] : 0.0;
+      const double x = k < d ? ((double)X[i * d + k] - ctr_.lo[k]) * ctr_.mul : 0.0;
       s.csum[i * dp + k] = x;
       s.cent[i * dp + k] = x;
       s.cent32[i * dp + k] = (float)x;
@@ -282,7 +283,7 @@ __global__ void k_layout_pos(State s, const T *X, const int32_t *perm, const uin
        p += (int64_t)gridDim.x * blockDim.x) {
     const int i = perm[p];
     for (int k = 0; k < dp; ++k) {
-      const double x = k < d ? (double)X[(int64_t)i * d + k] - ctr_.lo[k] : 0.0;
+      const double x = k < d ? ((double)X[(int64_t)i * d + k] - ctr_.lo[k]) * ctr_.mul : 0.0;
       s.q32[p * dp + k] = (float)x;
       s.q64[p * dp + k] = x;
       if (points) {
@@ -290,7 +291,8 @@ __global__ void k_layout_pos(State s, const T *X, const int32_t *perm, const uin
         // FP32 input stays unrounded (exact) in the FP32 copy; differences of
         // FP32 numbers then carry only relative rounding error
         s.p32[0][p * dp + k] =
-            s.pts32_exact ? (k < d ? (float)X[(int64_t)i * d + k] : 0.f) : (float)x;
+            s.pts32_exact ? (k < d ? (float)((double)X[(int64_t)i * d + k] * ctr_.mul) : 0.f)
+                          : (float)x;
       }
       if (s.linkage == LK_COMPLETE) {
         s.qblo[p * dp + k] = __double2float_rd(x);
@@ -311,12 +313,13 @@ __global__ void k_layout_pos(State s, const T *X, const int32_t *perm, const uin
 }
 
 // one instance's parameters and progress counters
-__global__ void k_inst_set(State s, int slot, float slack, float scale, float dpts, int rec,
-                           int act, int seq) {
+__global__ void k_inst_set(State s, int slot, float slack, float scale, float dpts, double unit,
+                           int rec, int act, int seq) {
   s.iseq[slot] = seq;
   s.islack[slot] = slack;
   s.iscale[slot] = scale;
   s.idpts[slot] = dpts;
+  s.iunit[slot] = unit;
   s.irec[slot] = rec;
   s.irecn[slot] = 0;
   s.iact[slot] = act;
@@ -1193,7 +1196,7 @@ __global__ void k_rec_gather(const State s, int m, const int32_t *perm, hac_merg
     hac_merge r;
     r.cid_a = s.m_a[v];
     r.cid_b = s.m_b[v];
-    r.height = s.m_h[v];
+    r.height = unit_height(s.m_h[v], s.iunit[0], s.linkage == LK_AVG2);
     r.size = s.m_size[v];
     out[i] = r;
     out_round[i] = s.m_round[v];
@@ -1296,6 +1299,7 @@ int alloc_state(hac_ctx *h) {
   A(s.islack, s.max_inst);
   A(s.iscale, s.max_inst);
   A(s.idpts, s.max_inst);
+  A(s.iunit, s.max_inst);
   A(s.irec, s.max_inst);
   A(s.irecn, s.max_inst);
   A(s.iact, s.max_inst);
@@ -1422,6 +1426,7 @@ int bits_for(int64_t maxval) {
 // Initial layout (Algorithm 1 initialisation): bounding box, recentring,
 // Morton keys, radix sort, permuted points and per-cluster state, the tree.
 // Host buffers are stack arrays, so hac_run_static can use it unchanged.
+// In the FP32 mode a copy that FP32 squares would overflow turns the run to FP64.
 template <typename T>
 int init_layout(hac_ctx *h, cudaStream_t st) {
   State &s = h->s;
@@ -1461,12 +1466,18 @@ int init_layout(hac_ctx *h, cudaStream_t st) {
     raw = std::max(raw, std::max(std::fabs(lo), std::fabs(hi)));
   }
   // the FP32 copy holds the input itself (FP32 input) or the recentred points
-  s.p32_max = s.pts32_exact ? raw : scale * (1.0 + 1e-6);
+  const double p32_max = s.pts32_exact ? raw : scale * (1.0 + 1e-6);
+  if (p32_max >= FP32_COORD_LIMIT) s.prec = HAC_PREC_F64;
+  const int ue = unit_exp(scale);
+  ctrp.mul = std::ldexp(1.0, -ue);
+  s.p32_max = p32_max * ctrp.mul;
+  scale *= ctrp.mul;
   mp.bits = std::min(21, 64 / d);
   s.abs_slack = std::max(scale, 1e-300) * std::ldexp(1.0, -18);
   s.coord_scale = (float)(scale * (1.0 + 1e-6));
   s.delta_pts = s.pts32_exact ? 0.f : 2.01f * 5.9604645e-8f * s.coord_scale * std::sqrt((float)d);
-  k_inst_set<<<1, 1, 0, st>>>(s, 0, (float)s.abs_slack, s.coord_scale, s.delta_pts, 0, (int)n, 0);
+  k_inst_set<<<1, 1, 0, st>>>(s, 0, (float)s.abs_slack, s.coord_scale, s.delta_pts, std::ldexp(1.0, ue),
+                              0, (int)n, 0);
   k_morton<T><<<grid_for(n, TPB), TPB, 0, st>>>(X, n, d, mp, h->keys[0], h->vals[0]);
   CK(cudaGetLastError());
   // a run that never searches the tree needs no spatial order; at few points
@@ -1677,7 +1688,8 @@ void fill_query_args(hac_ctx *h, QueryArgs &qa, int round, int K, int nterm) {
 bool use_brute(const hac_ctx *h) {
   const State &s = h->s;
   if (!closed_form(s.linkage) || s.prec != HAC_PREC_F32_RECHECK || s.max_inst != 1) return false;
-  // the screening's FP32 squares neither flush nor overflow
+  // the screening's FP32 squares neither flush nor overflow (false only for an extent
+  // of 0 or a subnormal one: unit_exp)
   if (!(s.coord_scale >= (float)FIN_SCALE_LO && s.coord_scale < (float)FIN_SCALE_HI)) return false;
   if (!h->own) return false;  // hac_run_static: no memory for the lists
   if (h->brute_env >= 0) return h->brute_env == 1 && (s.dp == 8 || s.dp == 16);
@@ -2267,7 +2279,6 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
   cudaEventRecord(e0.e, st);
   int rc = h->dt == HAC_F32 ? init_layout<float>(h, st) : init_layout<double>(h, st);
   if (rc) return rc;
-  if (s.p32_max >= FP32_COORD_LIMIT) s.prec = HAC_PREC_F64;  // FP32 would overflow
   cudaEventRecord(e1.e, st);
   CK(cudaEventSynchronize(e1.e));
   {
@@ -2547,6 +2558,7 @@ bool carve_state(hac_ctx &h, Carver &cv) {
   cv.take(&s.islack, 1);
   cv.take(&s.iscale, 1);
   cv.take(&s.idpts, 1);
+  cv.take(&s.iunit, 1);
   cv.take(&s.iseq, 1);
   cv.take(&s.done_list, 2);
   cv.take(&s.irec, 1);
@@ -2605,7 +2617,6 @@ int static_run(hac_ctx &h, const hac_opts &opt, cudaStream_t st, hac_merge *dev_
   if (rc || direct) return rc;
   rc = h.dt == HAC_F32 ? init_layout<float>(&h, st) : init_layout<double>(&h, st);
   if (rc) return rc;
-  if (s.p32_max >= FP32_COORD_LIMIT) s.prec = HAC_PREC_F64;  // FP32 would overflow
   RoundCtl ctl;  // no events: nothing is created here
   int rounds = 0;
   rc = run_rounds(&h, opt, st, ctl, nullptr, t0, &rounds);

@@ -20,9 +20,9 @@
 // hac_query.cuh (|D32 - D| <= delta + rho D, delta = 2.01 u M sqrt(d)
 // [* sqrt(w) for Ward]), U = least upper bound; a terminal whose second least
 // lower bound exceeds U has its winner, any other re-scores every candidate
-// within U in FP64.  Inputs whose recentred coordinates could overflow or
-// flush the FP32 squares (largest below 2^-30 or from 2^40) take the ordinary
-// rounds.
+// within U in FP64.  The coordinates' scale (unit_exp) keeps the FP32 squares from
+// overflow and flush; inputs without one (all points equal, subnormal extent) take
+// the ordinary rounds.
 //
 // "Direct" runs (n within the capacity) start from the input points: bounding
 // box, recentring and the singletons' state are made by the same kernel, and
@@ -312,7 +312,10 @@ __device__ bool fin_start(const FinArgs &a, const FinSm &m, double *s_box, float
     const double c = 0.5 * (s_box[k] + s_box[MAXD + k]);
     scale = fmax(scale, fmax(fabs(s_box[k] - c), fabs(s_box[MAXD + k] - c)));
   }
-  if (!(scale >= FIN_SCALE_LO && scale < FIN_SCALE_HI)) {
+  const int ue = unit_exp(scale);
+  const double mul = ldexp(1.0, -ue);
+  scale *= mul;
+  if (!(scale >= FIN_SCALE_LO && scale < FIN_SCALE_HI)) {  // all points equal, or subnormal
     if (cta_rank() == 0 && threadIdx.x == 0) s.ctr->fin_refused = 1;
     return false;
   }
@@ -324,11 +327,12 @@ __device__ bool fin_start(const FinArgs &a, const FinSm &m, double *s_box, float
 #pragma unroll
     for (int k = 0; k < D; ++k)
       m.x[k * a.Kc + i] =
-          k < d ? (float)((double)X[(size_t)i * d + k] - 0.5 * (s_box[k] + s_box[MAXD + k])) : 0.f;
+          k < d ? (float)(((double)X[(size_t)i * d + k] - 0.5 * (s_box[k] + s_box[MAXD + k])) * mul)
+                : 0.f;
   }
   for (int i = cta_rank() * FT + threadIdx.x; i < n; i += cta_count() * FT) {
     for (int k = 0; k < d; ++k) {
-      const double x = (double)X[(size_t)i * d + k] - 0.5 * (s_box[k] + s_box[MAXD + k]);
+      const double x = ((double)X[(size_t)i * d + k] - 0.5 * (s_box[k] + s_box[MAXD + k])) * mul;
       s.csum[(size_t)i * dp + k] = x;
       s.cent[(size_t)i * dp + k] = x;
       s.cent32[(size_t)i * dp + k] = (float)x;
@@ -343,6 +347,7 @@ __device__ bool fin_start(const FinArgs &a, const FinSm &m, double *s_box, float
   if (cta_rank() == 0 && threadIdx.x == 0) {
     s.irec[0] = 0;
     s.irecn[0] = 0;
+    s.iunit[0] = ldexp(1.0, ue);
   }
   return true;
 }
@@ -385,12 +390,13 @@ __device__ void fin_records(const State &s, int m, hac_merge *out, int32_t *out_
       }
       __syncthreads();
     }
+  const double unit = __ldcg(s.iunit);
   for (int i = threadIdx.x; i < m; i += FT) {
     const int v = idx[i];
     hac_merge r;
     r.cid_a = (int)(unsigned)ks[i];
     r.cid_b = __ldcg(&s.m_b[v]);
-    r.height = __longlong_as_double((long long)kh[i]);
+    r.height = unit_height(__longlong_as_double((long long)kh[i]), unit, s.linkage == LK_AVG2);
     r.size = (int)(ks[i] >> 32);
     out[i] = r;
     out_round[i] = __ldcg(&s.m_round[v]);

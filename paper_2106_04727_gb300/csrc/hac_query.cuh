@@ -780,7 +780,7 @@ struct Searcher {
       if (seed && __popc(m) > 1) {
         // nearest-looking candidate first: it usually settles the bound
         float v = ok ? d32 : INFINITY;
-        int who = lane;
+        int who = ok ? lane : lane + 32;  // an infinite v ties with the other lanes': they lose
         warp_argmin_f(v, who);
         unsigned long long k = KINF;
         int c = INT_MAX;
@@ -864,8 +864,9 @@ struct Searcher {
     }
     unsigned big = __ballot_sync(0xffffffffu, ok && !small);
     while (big) {
-      float v = (big >> lane) & 1u ? lb : INFINITY;
-      int who = lane;
+      const bool left = (big >> lane) & 1u;
+      float v = left ? lb : INFINITY;
+      int who = left ? lane : lane + 32;  // ties on infinity go to a candidate: the loop ends
       warp_argmin_f(v, who);
       big &= ~(1u << who);
       if (!pass(v)) break;  // remaining candidates have lb >= v

@@ -42,6 +42,7 @@ constexpr int SRV_ADMIT_MAX = 1024;  // requests admitted between two rounds
 struct AdmitInst {
   int base, n, off, slot, seq, bits;
   float slack, scale, dpts;               // the instance's pruning and error parameters
+  double mul, unit;                       // power of two for its coordinates, and its inverse
   double lo[MAXD], inv[MAXD], ctr[MAXD];  // Morton box and recentring offset
 };
 
@@ -53,6 +54,7 @@ __global__ void k_admit_inst(State s, const AdmitInst *ai, int na) {
     s.islack[a.slot] = a.slack;
     s.iscale[a.slot] = a.scale;
     s.idpts[a.slot] = a.dpts;
+    s.iunit[a.slot] = a.unit;
     s.irec[a.slot] = a.base;
     s.irecn[a.slot] = 0;
     s.iact[a.slot] = a.n;
@@ -78,7 +80,8 @@ __global__ void k_rec_pack(State s, const int4 *fin, int nf, int total, RecOut *
     }
     const int4 f = fin[lo];
     const int m = f.x + (i - f.z);
-    dst[i] = RecOut{s.m_a[m] - f.x, s.m_b[m] - f.x, s.m_size[m], s.m_round[m] - f.w, s.m_h[m]};
+    const double h = unit_height(s.m_h[m], s.iunit[s.inst[f.x]], s.linkage == LK_AVG2);
+    dst[i] = RecOut{s.m_a[m] - f.x, s.m_b[m] - f.x, s.m_size[m], s.m_round[m] - f.w, h};
   }
 }
 
@@ -132,9 +135,9 @@ __global__ void k_admit_layout(State s, const T *stage, int m, const AdmitInst *
     const int op = K + p;
     for (int k = 0; k < dp; ++k) {
       const double raw = k < d ? (double)stage[(size_t)i * d + k] : 0.0;
-      const double x = k < d ? raw - a.ctr[k] : 0.0;
+      const double x = k < d ? (raw - a.ctr[k]) * a.mul : 0.0;
       s.p64[pc][pp * dp + k] = x;
-      s.p32[pc][pp * dp + k] = s.pts32_exact ? (float)raw : (float)x;
+      s.p32[pc][pp * dp + k] = s.pts32_exact ? (float)(raw * a.mul) : (float)x;
       s.csum[(size_t)c * dp + k] = x;
       s.cent[(size_t)c * dp + k] = x;
       s.cent32[(size_t)c * dp + k] = (float)x;
@@ -147,7 +150,7 @@ __global__ void k_admit_layout(State s, const T *stage, int m, const AdmitInst *
     }
     double sq = 0.0;
     for (int k = 0; k < d; ++k) {
-      const double x = (double)stage[(size_t)i * d + k] - a.ctr[k];
+      const double x = ((double)stage[(size_t)i * d + k] - a.ctr[k]) * a.mul;
       sq += x * x;
     }
     s.csq[c] = sq;
@@ -406,6 +409,10 @@ int engine_admit(Engine &e, const std::vector<SrvReq *> &batch) {
       if (k < d)
         scale = std::max(scale, std::max(std::fabs(lo[k] - a.ctr[k]), std::fabs(hi[k] - a.ctr[k])));
     }
+    const int ue = unit_exp(scale);
+    a.mul = std::ldexp(1.0, -ue);
+    a.unit = std::ldexp(1.0, ue);
+    scale *= a.mul;
     a.slack = (float)(std::max(scale, 1e-300) * std::ldexp(1.0, -18));
     a.scale = (float)(scale * (1.0 + 1e-6));
     a.dpts = f32 ? 0.f : 2.01f * 5.9604645e-8f * a.scale * std::sqrt((float)d);
