@@ -548,6 +548,8 @@ int fin_pow2(int m) {
   return P;
 }
 constexpr int REC_BYTES = 20;  // sorted per record
+constexpr int FIN_REC_SMEM = FIN_MAX_K * REC_BYTES;
+static_assert(FIN_REC_SMEM <= FIN_SMEM, "a direct run's record sort fits the staged records' limit");
 
 template <int LK, int D>
 int launch_d(FinArgs &a, cudaStream_t st) {
@@ -584,8 +586,10 @@ int launch_lk_fin(FinArgs &a, cudaStream_t st) {
 
 int launch_cluster(const void *kern, int nct, int threads, size_t smem, void *args,
                    cudaStream_t st) {
+  // The limit belongs to the kernel, not to this call: always the same value, so that a
+  // launch of another thread is never left above it
   if (smem > 48 * 1024)
-    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FIN_SMEM));
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
@@ -611,8 +615,8 @@ int launch_cluster(const void *kern, int nct, int threads, size_t smem, void *ar
 
 int launch_rec_sort(const State &s, int m, hac_merge *out, int32_t *out_round, cudaStream_t st) {
   const size_t smem = (size_t)fin_pow2(m) * REC_BYTES;
-  if (smem > 48 * 1024)
-    CK(cudaFuncSetAttribute(k_rec_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > 48 * 1024)  // (one value for every call, as in launch_cluster)
+    CK(cudaFuncSetAttribute(k_rec_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, FIN_REC_SMEM));
   k_rec_sort<<<1, FT, smem, st>>>(s, m, out, out_round);
   CK(cudaGetLastError());
   return HAC_OK;
