@@ -1876,14 +1876,17 @@ int round_step(hac_ctx *h, cudaStream_t st, int round, int K, int nterm, RoundCt
     const int S = s.cache_slots;
     const size_t smem = (size_t)CM_WARPS * 5 * S * sizeof(CEntry);
     const int blocks = std::max(1, std::min(cdiv(npairs, CM_WARPS), device_sms() * 32));
-    // more than the default 48 KB of shared memory per block for large tables
+    // more than the default 48 KB of shared memory per block for large tables: the
+    // kernel's limit is set to the largest in every call, since other host threads
+    // launch under it too
+    constexpr int kMost = CM_WARPS * 5 * CACHE_MAX_SLOTS * (int)sizeof(CEntry);
     if (s.linkage == LK_COMPLETE) {
       CK(cudaFuncSetAttribute(k_cache_merge<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem));
+                              kMost));
       k_cache_merge<0><<<blocks, CM_WARPS * 32, smem, st>>>(s, npairs, round);
     } else {
       CK(cudaFuncSetAttribute(k_cache_merge<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem));
+                              kMost));
       k_cache_merge<1><<<blocks, CM_WARPS * 32, smem, st>>>(s, npairs, round);
     }
     k_gen_bump<<<grid_for(npairs, TPB), TPB, 0, st>>>(s, npairs);

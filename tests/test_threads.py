@@ -48,3 +48,17 @@ def test_one_launch_runs(lk):
     """Staged records of 1,600 to 4,000 clusters: 51 to 128 KB."""
     jobs = [_job(inputs.gaussian_mixture(n, 5, 6, seed=n), lk) for n in (1600, 4000, 2300, 3100)]
     assert _together(jobs, 150) == []
+
+
+def test_cache_updates(monkeypatch):
+    """256 slots a cluster take more than the default 48 KB, 8 and 64 do not."""
+    monkeypatch.setenv("HAC_DENSE_K", "0")
+    X = inputs.gaussian_mixture(1500, 2, 5, seed=3)
+    # (heights, and with them ties, depend on what the cache kept: sizes only)
+    jobs = []
+    for slots in (256, 8, 256, 64):
+        def run(slots=slots):
+            got = hac.cluster(X, "complete", cache_slots=slots)
+            assert got["size"][-1] == len(X)
+        jobs.append(run)
+    assert _together(jobs, 60) == []
