@@ -920,6 +920,9 @@ __global__ void __launch_bounds__(256) k_dense_nn(NNArgs a) {
     for (int p = lane; p < a.K; p += 32) {
       const unsigned long long x = (unsigned long long)__double_as_longlong(row[p]);
       if (!(x & SIGN) || (x & ~SIGN) > r.win) continue;
+      // a full list counts no further: 2^31 estimates can lie in the windows of
+      // 46,341 terminals, and a wrapped counter would pass as an index
+      if (*(volatile int32_t *)&a.ctr->nrq >= a.drq_cap) break;
       const int q = atomicAdd(&a.ctr->nrq, 1);
       if (q < a.drq_cap) {
         a.drq_a[q] = min(qi, p);

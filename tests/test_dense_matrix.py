@@ -90,3 +90,19 @@ def test_round_limits(lk):
             _check(got, want, 1e-5 if "precision" in kw else 1e-9)
     finally:
         hac.hac_destroy(h)
+
+
+def test_more_estimates_in_the_windows_than_a_counter_holds(monkeypatch):
+    """46,400 points whose FP32 distances all lie within the error term (set by one
+    point far away): 2.15 * 10^9 estimates are listed for an FP64 re-score, pass by
+    pass through a list of 4 * 10^6."""
+    n, d = 46_400, 16
+    monkeypatch.setenv("HAC_DENSE_K", str(n))
+    r = np.random.RandomState(11)
+    X = r.randint(0, 2, (n, d)) * 2.0**-25 + 2.0**-30 * r.uniform(size=(n, d))
+    X[0] = -1.0
+    h = hac.hac_create(X, "complete")
+    try:  # the first round lists them all
+        assert hac.hac_run(h, precision=hac.PREC_F32_RECHECK, max_rounds=1) == hac.HAC_ETIMEOUT
+    finally:
+        hac.hac_destroy(h)
