@@ -2206,11 +2206,15 @@ int run_impl(hac_ctx *h, const hac_opts *o) {
         (rc0 = dalloc(h, &s.cerr, cells)) || (rc0 = dalloc(h, &s.cpart, cells)))
       return rc0;
     if (!s.ins_i) {  // queue of evaluated pairs to insert (sized once per handle)
+      // (in one piece: a run that fails here leaves none of them set for the next)
       const int64_t cap = std::max<int64_t>(4 * h->n, 1 << 16);
-      if ((rc0 = dalloc(h, &s.ins_i, cap)) || (rc0 = dalloc(h, &s.ins_j, cap)) ||
-          (rc0 = dalloc(h, &s.ins_v, cap)) || (rc0 = dalloc(h, &s.ins_e, cap)) ||
-          (rc0 = dalloc(h, &s.cused, h->n)))
-        return rc0;
+      SlabAlloc m;
+      m.add(&s.ins_i, cap);
+      m.add(&s.ins_j, cap);
+      m.add(&s.ins_v, cap);
+      m.add(&s.ins_e, cap);
+      m.add(&s.cused, h->n);
+      if ((rc0 = m.commit(h))) return rc0;
       s.ins_cap = (int)cap;
     }
     if (!s.breq_i) {  // big-pair deferral buffers (sized once per handle)
