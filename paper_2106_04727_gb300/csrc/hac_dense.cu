@@ -666,8 +666,8 @@ __device__ __noinline__ double dist64(const double *x, const double *y, int d) {
 
 // The matrix of K singletons, straight from the points (position p is point p
 // of the layout): one thread per pair, no sums to collect by atomics.  The
-// distances are those of the sweeps (FP32: scaled coordinates, flush-to-zero
-// root; FP64: the same fma chain).  Bound by the 24-32 B written per pair, or
+// distances are those of the sweeps (FP32: scaled coordinates, for average the
+// flush-to-zero root; FP64: the same fma chain).  Bound by the 24-32 B written per pair, or
 // in FP64 by the square roots; the segmented sweep, which flushes every column
 // of every row through atomics when each point is a cluster of its own, took
 // 11 ms with its last pass at 20,001 points in 10-D, this 2.7.
@@ -717,8 +717,9 @@ __global__ void __launch_bounds__(32 * FT_Y) k_dense_single(State s, const float
         if (zero) {
           v = z;
         } else if (F32) {
-          // back to unscaled units (a power of two: exact)
-          const double m = (double)sqrt_approx_ftz((float)d2) * (double)inv_scl;
+          // the rounded root, as the evaluations of the searches take it; back to
+          // unscaled units (a power of two: exact)
+          const double m = (double)sqrtf((float)d2) * (double)inv_scl;
           v = __longlong_as_double((long long)((unsigned long long)__double_as_longlong(m) | SIGN));
         } else {
           v = sqrt((double)d2);

@@ -106,3 +106,18 @@ def test_more_estimates_in_the_windows_than_a_counter_holds(monkeypatch):
         assert hac.hac_run(h, precision=hac.PREC_F32_RECHECK, max_rounds=1) == hac.HAC_ETIMEOUT
     finally:
         hac.hac_destroy(h)
+
+
+def test_complete_estimates_are_correctly_rounded():
+    """Differences of points of [1, 2) on a line are FP32 numbers, and the rounded root
+    of their rounded square is they: every height that was not re-scored is the FP64
+    value plus the same bound."""
+    X = (1.0 + np.random.RandomState(4).uniform(size=(900, 1))).astype(np.float32)
+    got = hac.cluster(X, "complete", precision=hac.PREC_F32_RECHECK)
+    want = oracle.nnchain(X.astype(np.float64), "complete")
+    assert oracle.compare(got, want, rtol=1e-5)["ok"]
+    true = dict(zip(zip(want["a"].tolist(), want["b"].tolist()), want["h"]))
+    step = np.array([np.float64(h).view(np.int64) - np.float64(true[a, b]).view(np.int64)
+                     for a, b, h in zip(got["a"].tolist(), got["b"].tolist(), got["h"])])
+    assert np.count_nonzero(step) > 300
+    assert len(np.unique(step[step != 0])) == 1   # the bound is a step of the bit pattern
