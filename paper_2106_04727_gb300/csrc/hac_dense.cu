@@ -177,10 +177,10 @@ __device__ __forceinline__ U128 u128_shfl_xor(const U128 &v, int o) {
 
 // A finished sum is two words (lo, hi), the estimate flag in the top bit of hi.
 // The mean distance of an entry, one function everywhere so that equal sums
-// and sizes give equal means: the 128-bit sum as the nearest FP64 number (to
-// even), times 1 / size of the cluster with the lower matrix index, times 1 /
-// size of the other (reciprocals kept per matrix index: no FP64 division);
-// the sign bit set for an estimate.  The FP64 pipe (2 lanes per clock and SM)
+// and sizes give equal means, whichever cluster has which size: the 128-bit
+// sum as the nearest FP64 number (to even), times the product of 1 / size of
+// both (reciprocals kept per matrix index: no FP64 division); the sign bit
+// set for an estimate.  The FP64 pipe (2 lanes per clock and SM)
 // bounds every kernel that makes means, so the sum is converted by integer
 // instructions and two FP64 multiplications are left: the matrix rebuild at
 // 16,106 clusters took 1.90 ms with the seven FP64 instructions of two integer
@@ -213,8 +213,8 @@ __device__ __forceinline__ double sum_double(unsigned long long hi, unsigned lon
   return __longlong_as_double((long long)(((unsigned long long)(be - 1) << 52) + r));
 }
 
-__device__ __forceinline__ double entry_mean(const U128 &v, int e, double inv_lo, double inv_hi) {
-  const double m = sum_double(v.hi & ~TOP, v.lo, e) * inv_lo * inv_hi;
+__device__ __forceinline__ double entry_mean(const U128 &v, int e, double inv_a, double inv_b) {
+  const double m = sum_double(v.hi & ~TOP, v.lo, e) * (inv_a * inv_b);
   const unsigned long long b = (unsigned long long)__double_as_longlong(m);
   return __longlong_as_double((long long)(v.hi & TOP ? (b | SIGN) : b));
 }
@@ -1525,8 +1525,8 @@ __global__ void __launch_bounds__(DF_T, 1) k_tri_finish(TriArgs a) {
       for (int p = lane; p < K; p += 32) {
         const int r = s_slot[p];
         double v = p == self ? 0.0 : __ldcg(T + at(q, r));
-        // mean: 1 / size of the lower slot first, so both sides agree
-        if (LK == LK_AVERAGE) v = q < r ? v * iq * s_inv[r] : v * s_inv[r] * iq;
+        // mean, as entry_mean takes it
+        if (LK == LK_AVERAGE) v *= iq * s_inv[r];
         const unsigned long long k = (unsigned long long)__double_as_longlong(v);
         if (p != self && (k < bk || (k == bk && bp >= 0 && s_cid[p] < s_cid[bp]))) {
           bk = k;
