@@ -222,18 +222,23 @@ const char *hac_strerror(int code);
  * synchronisation that cudaMalloc/cudaFree can cause).
  *
  * Same dendrogram as hac_create + hac_run + hac_dendrogram on the same points
- * and options (with the dense matrix off, HAC_DENSE_K=0;
- * with it on, the same tree and heights within the precision mode's stated
- * bound), computed by the same kernels, but all working memory comes
- * from a fixed 6 MiB device array inside the library, which every GPU that
+ * and options: the same tree and heights within the precision mode's stated
+ * bound, and limits in opts change neither.  One thing can differ: average
+ * distances that tie up to the rounding of their FP64 sums.  With at most
+ * 1,280 points in HAC_PREC_F64 sums are exact as on hac_run's matrix, and
+ * the dendrogram is hac_run's bit for bit; otherwise rounds on the range-query
+ * search (here until that many clusters are left, in hac_run with
+ * HAC_DENSE_K=0) round sums in an order that depends on the layout, and such a
+ * tie may go either way.  All working memory comes
+ * from a fixed 16 MiB device array inside the library, which every GPU that
  * loads the library holds until the process exits.  No cudaMalloc, cudaFree
  * or other allocating call is made.  The pair-distance cache needs memory, so
  * opts->cache_slots is ignored (no cache, hence no GPU-wide big-pair
  * evaluation; in HAC_PREC_F64 complete and average linkage move to a packed
- * triangle of pair distances once it fits what is left of the array), and the HAC_* environment overrides that hac_create reads
- * (HAC_BIG_PAIRS, HAC_BIG_PAIRS_F64, HAC_WARP_BUDGET, HAC_BRUTE, HAC_DENSE_K) do
- * not apply;
- * these change speed only, never the result.  HAC_FLAG_NO_PRUNE is honoured.
+ * triangle of pair distances once at most 1,280 clusters are left, fewer where
+ * many points leave less of the array), and the HAC_* environment overrides
+ * that hac_create reads (HAC_BIG_PAIRS, HAC_BIG_PAIRS_F64, HAC_WARP_BUDGET,
+ * HAC_BRUTE, HAC_DENSE_K) do not apply.  HAC_FLAG_NO_PRUNE is honoured.
  *   dev_points  DEVICE pointer, row-major n x d of `dt`, on the current device;
  *               read only, owned by the caller.
  *   opts        may be NULL (defaults); opts->stream selects the stream

@@ -2042,10 +2042,11 @@ int run_rounds(hac_ctx *h, const hac_opts &opt, cudaStream_t st, RoundCtl &ctl, 
       continue;
     }
     if (h->tri && K <= h->tri_cap) {
-      rc = tri_finish(h, st, K, nterm, round, &c);
+      rc = tri_finish(h, st, K, nterm, round, finish_limit(opt, round), &c);
       if (rc) return rc;
-      if ((c.err & ~ERR_NONFINITE) || c.nactive != 1) return HAC_EINTERNAL;
-      K = 1;
+      if ((c.err & ~ERR_NONFINITE) || c.nactive >= K) return HAC_EINTERNAL;
+      K = c.nactive;
+      nterm = c.nterm;
       round += c.fin_rounds;
       ctl.searches += c.fin_searches;
       ctl.naive += c.fin_naive;
@@ -2490,7 +2491,10 @@ const char *hac_strerror(int code) {
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr size_t kStaticArenaBytes = (size_t)6 << 20;  // 6 MiB: room for n <= HAC_STATIC_MAX_N
+// 5.71 MB for the largest instance (n = HAC_STATIC_MAX_N, d > 8), the rest for the
+// packed triangle of average linkage in FP64: all 1,280 clusters it takes at most
+// up to that many points, 1,176 at HAC_STATIC_MAX_N in d > 8
+constexpr size_t kStaticArenaBytes = (size_t)16 << 20;
 static __device__ __align__(256) unsigned char g_static_arena[kStaticArenaBytes];
 
 // Device address of the arena on the current device, looked up on every
@@ -2673,15 +2677,13 @@ extern "C" int hac_run_static(const void *dev_points, int64_t n, int d, hac_dtyp
   Carver cv{arena, 0, kStaticArenaBytes, true};
   if (!carve_state(h, cv)) return HAC_EINVAL;
   // FP64 average / complete: the rest of the array holds the packed triangle of
-  // pair distances as soon as the active clusters' fits (not under a limit,
-  // which is checked between rounds)
-  if (!closed_form(h.s.linkage) && h.s.prec == HAC_PREC_F64 && !h.s.noprune && !opt.max_rounds &&
-      !(opt.timeout_s > 0)) {
+  // pair distances as soon as the active clusters' fits
+  if (!closed_form(h.s.linkage) && h.s.prec == HAC_PREC_F64 && !h.s.noprune) {
     const size_t at = (cv.off + 255) & ~(size_t)255;
-    const size_t cells = at < cv.cap ? (cv.cap - at) / sizeof(double) : 0;
+    const size_t cells = at < cv.cap ? (cv.cap - at) / tri_bytes(h.s.linkage) : 0;
     int k = TRI_MAX_K;
     while (k > 1 && (size_t)k * (k - 1) / 2 > cells) --k;
-    h.tri = (double *)(cv.base + at);
+    h.tri = cv.base + at;
     h.tri_cap = k;
   }
   const cudaStream_t st = (cudaStream_t)opt.stream;

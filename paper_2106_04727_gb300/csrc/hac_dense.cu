@@ -1410,20 +1410,29 @@ __global__ void __launch_bounds__(DF_T, 1) k_dense_finish(DFinArgs a) {
 // ---------------------------------------------------------------------------
 // FP64 rounds on a packed triangle (hac_run_static)
 // ---------------------------------------------------------------------------
-// The allocation-free entry point has a few MB to spare: once the active
-// clusters' packed upper triangle fits (8 B per pair: the sum of point
-// distances for average, the distance for complete), the FP64 mode fills it
-// from the points over the whole GPU and runs every remaining round in one
-// launch.  Without a cache its searches evaluate each big pair again in every
+// The allocation-free entry point has some MB to spare: once the active
+// clusters' packed upper triangle fits (average: the exact 128-bit sum of point
+// distances, 16 B per pair, as on the matrix, so that ties are broken alike;
+// complete: the distance, 8 B), the FP64 mode fills it from the points over the
+// whole GPU and runs every remaining round in one launch.  Without a cache its searches evaluate each big pair again in every
 // round, in one warp, and FP64 point pairs are bound by the SM's two-lane FP64
-// pipe: 1,024 points of 2-D average took 17.9 ms so, 0.68 here.
+// pipe: 1,024 points of 2-D average took 17.9 ms so, 0.60 here (0.66 with plain FP64 sums in a 6 MiB array).
 // Entries are patched in place: a round's survivors add (or take the larger
 // of) their partners' entries.
+template <int LK>
+using TriEntry = typename std::conditional<LK == LK_COMPLETE, double, ulonglong2>::type;
+
+__device__ __forceinline__ double tri_join(double x, double y) { return fmax(x, y); }
+__device__ __forceinline__ ulonglong2 tri_join(const ulonglong2 &x, const ulonglong2 &y) {
+  U128 s{x.x, x.y};
+  u128_add(s, U128{y.x, y.y});
+  return make_ulonglong2(s.lo, s.hi);
+}
 
 // one warp per pair of clusters
 template <int LK, int DP>
 __global__ void __launch_bounds__(256) k_tri_fill(State s, const int32_t *order, int K, int cur,
-                                                  double *tri_) {
+                                                  TriEntry<LK> *tri_) {
   const int lane = threadIdx.x & 31;
   const long long cells = (long long)K * (K - 1) / 2;
   const double *P = s.p64[cur];
@@ -1447,7 +1456,8 @@ __global__ void __launch_bounds__(256) k_tri_fill(State s, const int32_t *order,
       sa = sb;
       sb = x;
     }
-    double acc = 0.0;
+    double far2 = 0.0;
+    U128 acc{0ull, 0ull};
     for (int u = single ? 0 : lane; u < na; u += 32) {
       double x[DP];
 #pragma unroll
@@ -1462,19 +1472,24 @@ __global__ void __launch_bounds__(256) k_tri_fill(State s, const int32_t *order,
           }
         }
         if (LK == LK_COMPLETE)
-          acc = fmax(acc, d2);
+          far2 = fmax(far2, d2);
         else
-          acc += sqrt(d2);
+          u128_add(acc, fx_of(sqrt(d2), s.dexp));
       }
     }
     if (!single) {
       for (int o = 16; o; o >>= 1) {
-        const double y = __shfl_xor_sync(0xffffffffu, acc, o);
-        acc = LK == LK_COMPLETE ? fmax(acc, y) : acc + y;
+        if (LK == LK_COMPLETE)
+          far2 = fmax(far2, __shfl_xor_sync(0xffffffffu, far2, o));
+        else
+          u128_add(acc, u128_shfl_xor(acc, o));
       }
     }
     if (single || lane == 0) {
-      tri_[tri(i, j, K)] = LK == LK_COMPLETE ? sqrt(acc) : acc;
+      if constexpr (LK == LK_COMPLETE)
+        tri_[tri(i, j, K)] = sqrt(far2);
+      else
+        tri_[tri(i, j, K)] = make_ulonglong2(acc.lo, acc.hi);
       pp += (unsigned long long)na * nb;
     }
   }
@@ -1484,36 +1499,41 @@ __global__ void __launch_bounds__(256) k_tri_fill(State s, const int32_t *order,
 
 struct TriArgs {
   State s;
-  int K, nterm, round;
-  const int32_t *order;
-  double *tri;
+  int K, nterm, round, rounds_max;  // rounds to run at most (0 = to the end)
+  int K0;                           // clusters when the triangle was filled
+  int32_t *order;
+  void *tri;
 };
 
 constexpr int TRI_PER = (TRI_MAX_K + DF_T - 1) / DF_T;
 
 template <int LK>
 __global__ void __launch_bounds__(DF_T, 1) k_tri_finish(TriArgs a) {
-  // by position in the active list: cid, slot (position at the start); by slot:
-  // 1 / size and the partner of this round's merge (-1 none, -2 retired now)
+  // by position in the active list: cid, slot (position when the triangle was
+  // filled; the cid's pos, which is not rewritten here); by slot: 1 / size and the
+  // partner of this round's merge (-1 none)
   __shared__ int s_cid[TRI_MAX_K], s_slot[TRI_MAX_K], s_term[TRI_MAX_K], s_part[TRI_MAX_K];
   __shared__ double s_inv[TRI_MAX_K];
   __shared__ int ws[DF_W];
   const State &s = a.s;
-  const int rank = df_rank(), nct = df_count(), K0 = a.K;
+  const int rank = df_rank(), nct = df_count(), K0 = a.K0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int K = a.K, nterm = a.nterm, round = a.round;
-  double *T = a.tri;
+  TriEntry<LK> *T = (TriEntry<LK> *)a.tri;
   for (int p = threadIdx.x; p < K; p += DF_T) {
-    const int c = a.order[p];
+    const int c = a.order[p], q = s.pos[c];
     s_cid[p] = c;
-    s_slot[p] = p;
-    s_inv[p] = 1.0 / (double)s.csize[c];
+    s_slot[p] = q;
+    s_part[q] = p;  // for the terminals' positions
+    s_inv[q] = 1.0 / (double)s.csize[c];
   }
-  for (int t = threadIdx.x; t < nterm; t += DF_T) s_term[t] = s.pos[s.term[t]];
+  __syncthreads();
+  for (int t = threadIdx.x; t < nterm; t += DF_T) s_term[t] = s_part[s.pos[s.term[t]]];
   __syncthreads();
   auto at = [&](int x, int y) -> size_t { return x < y ? tri(x, y, K0) : tri(y, x, K0); };
   long long searches = 0, naive = 0;
-  while (K > 1) {
+  const int round_end = a.rounds_max > 0 ? round + a.rounds_max : INT_MAX;
+  while (K > 1 && round < round_end) {
     searches += nterm;
     naive += (long long)nterm * (K - 1);
     for (int t = rank * DF_W + wid; t < nterm; t += nct * DF_W) {
@@ -1524,11 +1544,16 @@ __global__ void __launch_bounds__(DF_T, 1) k_tri_finish(TriArgs a) {
 #pragma unroll 4
       for (int p = lane; p < K; p += 32) {
         const int r = s_slot[p];
-        double v = p == self ? 0.0 : __ldcg(T + at(q, r));
-        // mean, as entry_mean takes it
-        if (LK == LK_AVERAGE) v *= iq * s_inv[r];
+        if (p == self) continue;
+        double v;
+        if constexpr (LK == LK_COMPLETE) {
+          v = __ldcg(T + at(q, r));
+        } else {
+          const ulonglong2 u = __ldcg(T + at(q, r));
+          v = entry_mean(U128{u.x, u.y}, s.dexp, iq, s_inv[r]);
+        }
         const unsigned long long k = (unsigned long long)__double_as_longlong(v);
-        if (p != self && (k < bk || (k == bk && bp >= 0 && s_cid[p] < s_cid[bp]))) {
+        if ((k < bk || (k == bk && bp >= 0 && s_cid[p] < s_cid[bp]))) {
           bk = k;
           bp = p;
         }
@@ -1623,13 +1648,8 @@ __global__ void __launch_bounds__(DF_T, 1) k_tri_finish(TriArgs a) {
       if (p >= K2) continue;
       const int y = s_slot[p], d = s_part[y];
       if (y == x || (d >= 0 && y < x)) continue;  // both merged: the lower slot's warp does it
-      double v = __ldcg(T + at(x, y)), u = __ldcg(T + at(b, y));
-      v = LK == LK_COMPLETE ? fmax(v, u) : v + u;
-      if (d >= 0) {
-        const double g = __ldcg(T + at(x, d)), h = __ldcg(T + at(b, d));
-        u = LK == LK_COMPLETE ? fmax(g, h) : g + h;
-        v = LK == LK_COMPLETE ? fmax(v, u) : v + u;
-      }
+      TriEntry<LK> v = tri_join(__ldcg(T + at(x, y)), __ldcg(T + at(b, y)));
+      if (d >= 0) v = tri_join(v, tri_join(__ldcg(T + at(x, d)), __ldcg(T + at(b, d))));
       T[at(x, y)] = v;
     }
     K = K2;
@@ -1637,7 +1657,12 @@ __global__ void __launch_bounds__(DF_T, 1) k_tri_finish(TriArgs a) {
     ++round;
     df_sync();
   }
-  if (rank != 0 || threadIdx.x != 0) return;
+  if (rank != 0) return;
+  if (K > 1) {  // stopped by the round limit: the lists go back
+    for (int p = threadIdx.x; p < K; p += DF_T) a.order[p] = s_cid[p];
+    for (int t = threadIdx.x; t < nterm; t += DF_T) s.term[t] = s_cid[s_term[t]];
+  }
+  if (threadIdx.x != 0) return;
   s.ctr->nactive = K;
   s.ctr->nterm = nterm;
   s.ctr->nmerges += a.K - K;
@@ -1883,6 +1908,14 @@ int64_t dense_default(int64_t n, int d, int linkage, int prec) {
   return k;
 }
 
+// unit of the fixed-point sums: (n/2)^2 x the largest point distance < 2^126 units
+void set_sum_unit(hac_ctx *h) {
+  State &s = h->s;
+  const double dmax = 2.0 * (double)s.coord_scale * std::sqrt((double)s.d) * (1.0 + 1e-5);
+  const double smax = 0.25 * (double)h->lay_n * (double)h->lay_n * dmax;
+  s.dexp = smax > 0.0 ? (int)std::floor(std::log2(smax)) + 1 - 126 : -1000;
+}
+
 // Complete linkage keeps the whole matrix only from the first round on (at
 // most the threshold's points); average linkage switches in mid-run too.
 bool dense_allowed(const hac_ctx *h, int K) {
@@ -1907,10 +1940,7 @@ int dense_maybe_enter(hac_ctx *h, cudaStream_t st, int K, RoundCtl &ctl) {
   if (!dense_reserve(h, K)) return 0;
   s.dk = K;
   s.dld = dense_ld(K);
-  // unit of the fixed-point sums: (n/2)^2 x the largest point distance < 2^126 units
-  const double dmax = 2.0 * (double)s.coord_scale * std::sqrt((double)s.d) * (1.0 + 1e-5);
-  const double smax = 0.25 * (double)h->lay_n * (double)h->lay_n * dmax;
-  s.dexp = smax > 0.0 ? (int)std::floor(std::log2(smax)) + 1 - 126 : -1000;
+  set_sum_unit(h);
   // the FP32 copy scaled by 2^k toward |coordinate| <= 2^40 (squared
   // distances stay below 2^86 for d <= 16; k >= 0 keeps the scaling exact)
   int k = 0;
@@ -2090,29 +2120,44 @@ int dense_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64
   return HAC_OK;
 }
 
-// Every remaining round of an FP64 run on the packed triangle at h->tri
-// (room for h->tri_cap clusters); the counters come back in *c.
-int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, Counters *c) {
+size_t tri_bytes(int linkage) {
+  return linkage == LK_COMPLETE ? sizeof(TriEntry<LK_COMPLETE>) : sizeof(TriEntry<LK_AVERAGE>);
+}
+
+// The remaining rounds (at most `limit` of them, 0 = all) of an FP64 run on the
+// packed triangle at h->tri (room for h->tri_cap clusters), which the first call
+// fills; the counters come back in *c.
+int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64_t limit,
+               Counters *c) {
   State &s = h->s;
-  const int32_t *order = s.order[h->ocur];
+  int32_t *order = s.order[h->ocur];
   const int g = device_sms() * 8;
   const bool comp = s.linkage == LK_COMPLETE;
 #define TRI_FILL(DP)                                                                      \
-  (comp ? k_tri_fill<LK_COMPLETE, DP><<<g, 256, 0, st>>>(s, order, K, h->pcur, h->tri)    \
-        : k_tri_fill<LK_AVERAGE, DP><<<g, 256, 0, st>>>(s, order, K, h->pcur, h->tri))
-  switch (s.dp) {
-    case 2: TRI_FILL(2); break;
-    case 4: TRI_FILL(4); break;
-    case 8: TRI_FILL(8); break;
-    default: TRI_FILL(16);
+  (comp ? k_tri_fill<LK_COMPLETE, DP><<<g, 256, 0, st>>>(                                 \
+              s, order, K, h->pcur, (TriEntry<LK_COMPLETE> *)h->tri)                      \
+        : k_tri_fill<LK_AVERAGE, DP><<<g, 256, 0, st>>>(                                  \
+              s, order, K, h->pcur, (TriEntry<LK_AVERAGE> *)h->tri))
+  if (!h->tri_k0) {
+    h->tri_k0 = K;
+    set_sum_unit(h);
+    switch (s.dp) {
+      case 2: TRI_FILL(2); break;
+      case 4: TRI_FILL(4); break;
+      case 8: TRI_FILL(8); break;
+      default: TRI_FILL(16);
+    }
+    CK(cudaGetLastError());
+    h->launches += 1;
   }
 #undef TRI_FILL
-  CK(cudaGetLastError());
   TriArgs a{};
   a.s = s;
   a.K = K;
   a.nterm = nterm;
   a.round = round;
+  a.rounds_max = (int)std::min<int64_t>(limit, INT32_MAX / 2);
+  a.K0 = h->tri_k0;
   a.order = order;
   a.tri = h->tri;
   const int nct = K <= 64 ? 1 : K <= 200 ? 8 : 16;
@@ -2120,7 +2165,7 @@ int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, Counter
                                : (const void *)k_tri_finish<LK_AVERAGE>,
                           nct, DF_T, 0, &a, st);
   if (rc) return rc;
-  h->launches += 2;
+  h->launches += 1;
   CK(cudaMemcpyAsync(c, s.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return HAC_OK;

@@ -164,8 +164,9 @@ struct hac_ctx {
   int64_t n_merges = 0;
   hac_stats_t st{};
   // hac_run_static: memory for the packed triangle of up to tri_cap clusters
-  double *tri = nullptr;
-  int tri_cap = 0;
+  // (filled once, from tri_k0 clusters)
+  void *tri = nullptr;
+  int tri_cap = 0, tri_k0 = 0;
   hac_merge *dout = nullptr;        // canonical dendrogram (device)
   int32_t *dout_round = nullptr;
 };
@@ -324,8 +325,11 @@ int dense_update(hac_ctx *h, cudaStream_t st, int round, int Kold, int K);
 int dense_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64_t limit,
                  Counters *c);
 
-// FP64 average / complete: every remaining round on the packed triangle
-int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, Counters *c);
+// FP64 average / complete: the remaining rounds on the packed triangle, at most
+// `limit` of them (0 = all); its bytes per pair
+int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64_t limit,
+               Counters *c);
+size_t tri_bytes(int linkage);
 
 // points moved so that every cluster is one segment again, if they are not
 int relayout_if_stale(hac_ctx *h, cudaStream_t st);

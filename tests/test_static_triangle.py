@@ -64,3 +64,19 @@ def test_limits_and_no_prune(lk):
     Y = X.copy()
     Y[5, 1] = np.inf
     assert _static(Y, lk)[0] == hac.HAC_EINVAL
+
+
+@pytest.mark.parametrize("lk", ["complete", "average"])
+@pytest.mark.parametrize("n,d,levels", [(201, 3, 9), (201, 5, 4), (700, 8, 4), (900, 2, 9),
+                                        (1100, 2, 40), (1280, 1, 500)])
+def test_ties_as_on_the_matrix(lk, n, d, levels):
+    """Exact sums: lattice points' many tied distances give the tree and the heights of
+    hac_run's matrix bit for bit, whatever limits the call carries."""
+    X = inputs.lattice(n, d, seed=n, levels=levels).astype(np.float64)
+    want = hac.cluster(X, lk)
+    assert want["stats"]["dense_k"] == n
+    for opts in ({}, dict(timeout_s=60.0), dict(max_rounds=n)):
+        rc, got = _static(X, lk, **opts)
+        assert rc == hac.HAC_OK
+        for f in ("a", "b", "h", "size"):
+            assert np.array_equal(got[f], want[f]), (f, opts)
