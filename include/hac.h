@@ -235,8 +235,9 @@ const char *hac_strerror(int code);
  * or other allocating call is made.  The pair-distance cache needs memory, so
  * opts->cache_slots is ignored (no cache, hence no GPU-wide big-pair
  * evaluation; in HAC_PREC_F64 complete and average linkage move to a packed
- * triangle of pair distances once at most 1,280 clusters are left, fewer where
- * many points leave less of the array), and the HAC_* environment overrides
+ * triangle of pair distances once at most 1,280 clusters are left, 1,024 in
+ * complete linkage of more points in d <= 8, fewer where many points leave less
+ * of the array), and the HAC_* environment overrides
  * that hac_create reads (HAC_BIG_PAIRS, HAC_BIG_PAIRS_F64, HAC_WARP_BUDGET,
  * HAC_BRUTE, HAC_DENSE_K) do not apply.  HAC_FLAG_NO_PRUNE is honoured.
  *   dev_points  DEVICE pointer, row-major n x d of `dt`, on the current device;

@@ -2682,6 +2682,9 @@ extern "C" int hac_run_static(const void *dev_points, int64_t n, int d, hac_dtyp
     const size_t at = (cv.off + 255) & ~(size_t)255;
     const size_t cells = at < cv.cap ? (cv.cap - at) / tri_bytes(h.s.linkage) : 0;
     int k = TRI_MAX_K;
+    // (complete linkage prunes well in low dimension: entered in mid-run, 4,096 points
+    // in 3-D took 3.70 ms from 1,280 clusters and 3.38 from 1,024)
+    if (lk == HAC_COMPLETE && d <= 8 && n > TRI_MAX_K) k = 1024;
     while (k > 1 && (size_t)k * (k - 1) / 2 > cells) --k;
     h.tri = cv.base + at;
     h.tri_cap = k;
