@@ -81,3 +81,26 @@ def test_limits_and_bad_input(lk):
         assert hac.hac_run(h) == hac.HAC_EINVAL
     finally:
         hac.hac_destroy(h)
+
+
+@pytest.mark.parametrize("lk", LKS)
+@pytest.mark.parametrize("n,d,one", [(4096, 8, True), (3936, 9, True), (3936, 10, True),
+                                     (3937, 10, False), (3392, 11, True), (3392, 12, True),
+                                     (3393, 12, False), (2688, 13, True), (2689, 13, False)])
+def test_capacities(lk, n, d, one):
+    """The most points of a run that is one launch, by dimension, and one more; the
+    allocation-free entry point on both sides too."""
+    torch = pytest.importorskip("torch")
+    X = inputs.gaussian_mixture(n, d, 6, seed=n + d)
+    want = oracle.rounds(X.astype(np.float64), lk)
+    got = hac.cluster(X, lk, precision=hac.PREC_F32_RECHECK)
+    _check(got, want)
+    assert (got["stats"]["kernel_launches"] == 1) == one
+    src = torch.from_numpy(X).cuda()
+    out = torch.zeros((n - 1) * 4, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    for prec in (hac.PREC_F64, hac.PREC_F32_RECHECK):
+        assert hac.hac_run_static(src.data_ptr(), n, d, X.dtype, lk, out.data_ptr(), n - 1,
+                                  precision=prec) == hac.HAC_OK
+        c = oracle.compare(hac.result_dict(out.cpu().numpy().view(hac.MERGE_DTYPE)), want, rtol=1e-9)
+        assert c["ok"], c
