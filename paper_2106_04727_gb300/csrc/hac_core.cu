@@ -13,6 +13,10 @@
 //                               k_tg_*: rebuild the range-query tree
 #include "hac_impl.cuh"
 
+#include <errno.h>
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include <algorithm>
 #include <type_traits>
 #include <chrono>
@@ -2394,18 +2398,25 @@ int hac_run(hac_t h, const hac_opts *opts) {
 
 // Pages of a caller's buffer that nothing has touched yet are made by the CPU
 // before the copy: the copy engine's own faults on them take some 50 us a page
-// (32 MB of fresh memory: 26 ms, against 1.0 to touch and 0.3 to copy).  The
-// contents stay: the copy may still fail.
+// (32 MB of fresh memory: 26 ms; 0.9 this way, 0.3 of it the copy).  The contents
+// stay, since the copy may still fail: the kernel is asked for writable pages.  (An
+// atomic that adds nothing, the fallback of kernels before 5.14, faults twice on a
+// fresh private page, once to read it: 10^7 merges 97 ms more.)
 static void touch_pages(void *p, size_t bytes) {
-  constexpr size_t kPage = 4096, kAlone = (size_t)8 << 20;
+  // (320 MB with 1 / 4 / 8 / 16 threads: 9.4 / 3.6 / 4.6 / 6.4 ms)
+  constexpr size_t kPage = 4096, kAlone = (size_t)8 << 20, kThreads = 4;
   if (bytes < ((size_t)1 << 20)) return;
   auto touch = [](unsigned char *b, unsigned char *e) {
-    for (; b < e; b += kPage) __atomic_fetch_or(b, 0, __ATOMIC_RELAXED);  // a write, no change
+    constexpr int kPopulateWrite = 23;  // MADV_POPULATE_WRITE
+    if (b >= e) return;
+    unsigned char *lo = b - (uintptr_t)b % (uintptr_t)sysconf(_SC_PAGESIZE);
+    if (madvise(lo, (size_t)(e - lo), kPopulateWrite) == 0 || errno != EINVAL) return;
+    for (; b < e; b += kPage) __atomic_fetch_or(b, 0, __ATOMIC_RELAXED);
   };
   unsigned char *b = (unsigned char *)p;
-  const int parts = (int)std::min<size_t>(8, (bytes + kAlone - 1) / kAlone);
+  const int parts = (int)std::min<size_t>(kThreads, (bytes + kAlone - 1) / kAlone);
   const size_t step = (bytes / parts + kPage) / kPage * kPage;
-  std::thread thr[8];
+  std::thread thr[kThreads];
   int started = 1;
   try {
     for (; started < parts; ++started)

@@ -36,8 +36,9 @@ def test_touching_changes_nothing(tmp_path):
     a = text.index("static void touch_pages(")
     body = text[a:text.index("\n}\n", a) + 3]
     src = tmp_path / "touch.cpp"
-    src.write_text("#include <algorithm>\n#include <cstddef>\n#include <cstdio>\n"
-                   "#include <thread>\n#include <vector>\n" + body + MAIN)
+    src.write_text("#include <errno.h>\n#include <sys/mman.h>\n#include <unistd.h>\n"
+                   "#include <algorithm>\n#include <cstddef>\n#include <cstdint>\n"
+                   "#include <cstdio>\n#include <thread>\n#include <vector>\n" + body + MAIN)
     exe = tmp_path / "touch"
     r = subprocess.run([CXX, "-O2", "-std=c++17", "-pthread", str(src), "-o", str(exe)],
                        capture_output=True, text=True)
