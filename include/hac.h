@@ -176,9 +176,10 @@ int hac_create_device(const void *dev_points, int64_t n, int d, hac_dtype dt, ha
  * half of the device memory free when the run starts.  Complete linkage runs
  * on such a matrix (16 bytes per entry) from the first round on if it has at
  * most K points: 24,576 to 32,768 by d and precision, capped the same way.  A
- * run that starts on the matrix takes no cache.  Ward and avg-2 runs of at most
- * 4,096 points (d <= 10; 2,688 in 16-D) take no matrix and no tree either: all
- * their rounds are one launch.  The environment variable HAC_DENSE_K,
+ * run that starts on the matrix takes no cache.  The matrix stays with the handle
+ * until hac_destroy.  Ward and avg-2 runs of at most 4,096 points (d <= 8; 3,936
+ * in d <= 10, 3,392 in d <= 12, 2,688 above) take no matrix and no tree either:
+ * all their rounds are one launch.  The environment variable HAC_DENSE_K,
  * read at hac_create, sets it instead (0 = never).  opts may be NULL (defaults).  Blocks until done.  May be called
  * again on the same handle: each call recomputes from the stored points.
  * HAC_ETIMEOUT if a limit in opts is hit (the handle stays usable). */
@@ -198,7 +199,10 @@ int hac_dendrogram(hac_t h, hac_merge *out, int64_t cap, int64_t *n_written);
  * same order.  Same errors as hac_dendrogram. */
 int hac_merge_rounds(hac_t h, int32_t *out, int64_t cap, int64_t *n_written);
 
-/* Counters and phase times of the last hac_run (paper: Section 6, analysis of
+/* Rounds that run together in one launch (a whole Ward or avg-2 run of few points,
+ * the last rounds of any run) are not split into phases: their time is in ms_nn,
+ * and rechecks and ms_query do not count them.
+ * Counters and phase times of the last hac_run (paper: Section 6, analysis of
  * the framework -- point_pairs is the count of distance computations the
  * paper calls D, cluster_pairs and the search counters its range-query
  * statistics).  HAC_EINVAL for a NULL handle or out. */

@@ -16,7 +16,11 @@
 //                eps = 1.03 * 2^-10: each FP16 rounding is within 2^-11 of its
 //                coordinate, so the product sum is within (2^-10 + 2^-22)
 //                ||x|| ||y|| <= (2^-11 + 2^-23)(nx + ny), and the FP32
-//                accumulation within 2^-18 of that.  A pair whose bound is
+//                accumulation within 2^-18 of that.  (A scaled coordinate below
+//                2^-14 is a subnormal FP16 number, off by up to 2^-25 and not by
+//                2^-11 of itself: against a coordinate above 2^-9 the spare 0.03 of
+//                eps covers that, else the delta added to the threshold's root, at
+//                least 2^-12 sqrt(d) here.)  A pair whose bound is
 //                within the terminal's threshold is scored in FP32 exactly as
 //                the search does (|D32 - D| <= delta + rho D) and, if its lower
 //                bound is within U, goes on the terminal's list;

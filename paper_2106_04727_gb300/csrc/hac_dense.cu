@@ -28,9 +28,10 @@
 //
 // Exact sums.  Every entry is kept as the sum of its point distances in
 // 128-bit fixed point (unit 2^e, chosen per instance so that (n/2)^2 times the
-// largest point distance stays below 2^126 units; stored as four 32-bit limbs
-// in 64-bit words, so atomic additions need no carry), next to the mean
-// distance that sum gives in FP64.  Integer addition is exact and associative, so:
+// largest point distance stays below 2^126 units), two 64-bit words, next to the
+// mean distance that sum gives in FP64.  While the sweep or a re-score collects a
+// sum it is four 32-bit limbs in 64-bit words, so that its atomic additions need
+// no carry.  Integer addition is exact and associative, so:
 //   * tiles can add into a cell with atomics in any order and the run is
 //     deterministic;
 //   * the Lance-Williams update of average linkage is the exact addition of
@@ -109,7 +110,7 @@ __device__ __forceinline__ void u128_add(U128 &a, const U128 &b) {
   a.lo = lo;
 }
 
-// A stored sum is four 64-bit words, each the sum of one 32-bit limb of
+// A sum being collected is four 64-bit words, each the sum of one 32-bit limb of
 // every addend (w0 + w1 2^32 + w2 2^64 + w3 2^96), so additions need no
 // carries and go out as fire-and-forget atomics; 2^32 additions per word
 // cannot overflow.  The estimate flag is the top bit of w3 (sums stay below
@@ -2100,6 +2101,8 @@ int dense_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64
                    : (!f32 ? k_dense_finish<LK_AVERAGE, 0>
                            : intb ? k_dense_finish<LK_AVERAGE, 2> : k_dense_finish<LK_AVERAGE, 1>);
   CK(cudaMemsetAsync(&s.ctr->fin_refused, 0, sizeof(int32_t), st));
+  // (whole 3-D runs, ms, with 1 / 4 / 8 / 16 blocks: average 64 clusters 0.277 / 0.269 /
+  // 0.270 / 0.271, 200 0.413 / 0.351 / 0.341 / 0.333, 800 1.62 / 0.75 / 0.61 / 0.53)
   const int nct = K <= 64 ? 1 : K <= 200 ? 8 : 16;
   int rc = launch_cluster((const void *)kern, nct, DF_T, 0, &a, st);
   if (rc) return rc;
@@ -2160,6 +2163,8 @@ int tri_finish(hac_ctx *h, cudaStream_t st, int K, int nterm, int round, int64_t
   a.K0 = h->tri_k0;
   a.order = order;
   a.tri = h->tri;
+  // (static calls in 3-D, ms, with 1 / 4 / 8 / 16 blocks: average 64 clusters 0.266 / 0.263
+  // / 0.266 / 0.266, 200 0.410 / 0.333 / 0.327 / 0.316, 800 1.89 / 0.87 / 0.70 / 0.61)
   const int nct = K <= 64 ? 1 : K <= 200 ? 8 : 16;
   int rc = launch_cluster(comp ? (const void *)k_tri_finish<LK_COMPLETE>
                                : (const void *)k_tri_finish<LK_AVERAGE>,

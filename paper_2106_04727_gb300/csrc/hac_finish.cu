@@ -560,8 +560,11 @@ int launch_d(FinArgs &a, cudaStream_t st) {
   if (a.out) {  // the record sort reuses it
     smem = std::max(smem, (size_t)fin_pow2(a.n_rec) * REC_BYTES);
   }
-  // blocks: a search is K / 32 steps of one warp, so few clusters need few
-  // blocks (a barrier of one block is cheaper than the cluster's)
+  // blocks: a search is K / 32 steps of one warp, so few clusters need few blocks, and
+  // the lines leave the other SMs free where more bring nothing (whole runs, ms, with
+  // 1 / 4 / 8 / 16 blocks: 2-D Ward 96 clusters 0.192 / 0.188 / 0.188 / 0.189, 320 0.286 /
+  // 0.261 / 0.262 / 0.254, 640 0.434 / 0.335 / 0.322 / 0.312, 2,000 1.52 / 0.73 / 0.59 /
+  // 0.53; 16-D 2,000 5.2 / 2.2 / 1.8 / 1.5)
   const int nct = a.K <= 96 ? 1 : a.K <= 320 ? 4 : a.K <= 640 ? 8 : 16;
   return launch_cluster((const void *)kern, nct, FT, smem, &a, st);
 }

@@ -361,11 +361,11 @@ __host__ __device__ inline int fin_cap(int d) {
 }
 
 // The same for rounds on the dense matrix (hac_dense.cu): at most DFIN_K active
-// clusters, one list entry per thread of a block.
-#ifndef HAC_DFIN_K
-#define HAC_DFIN_K 1024
-#endif
-constexpr int DFIN_K = HAC_DFIN_K;
+// clusters, one list entry per thread of a block.  Whole 5-D runs, ms, with the one
+// launch from 0 (never) / 256 / 512 / 1,024 clusters: complete FP64 of 1,000 points
+// 2.35 / 1.07 / 0.82 / 0.54, average FP32 of 8,000 points 8.00 / 5.63 / 5.10 / 4.69;
+// more than 1,024 would take two entries a thread and more shared memory.
+constexpr int DFIN_K = 1024;
 // FP64 rounds on a packed triangle (hac_run_static's spare memory)
 constexpr int TRI_MAX_K = 1280;
 
@@ -384,7 +384,10 @@ cudaError_t launch_gsearch(const QueryArgs &a, int prec, cudaStream_t s);
 #ifndef HAC_GS_WIDE
 #define HAC_GS_WIDE 40000
 #endif
-constexpr int GS_WIDE = HAC_GS_WIDE;  // terminals from which a group is 32 (else 8)
+// terminals from which a group is 32 in d <= 2 and 8 above (below: 4).  The line is
+// flat (whole Ward runs, ms, at 20,000 / 40,000 / 80,000): 2-D 30,000 points 3.22 / 3.16
+// / 3.18, 60,000 4.13 / 4.01 / 3.97, 10^6 avg-2 10.8 / 10.7 / 10.5; 5-D no difference
+constexpr int GS_WIDE = HAC_GS_WIDE;
 
 // the same search done exhaustively, screened by tensor-core products of the
 // cluster records (hac_brute.cu): closed-form linkages, FP32 + FP64 re-score,

@@ -31,7 +31,10 @@ search), HAC_QMINB / HAC_QMINB_COMPLETE (its resident blocks per SM, which
 bound its registers; the second for complete linkage),
 HAC_Q_OUTLINE (1: its warp-wide pair evaluations compiled out of line),
 HAC_BR_T / HAC_BR_C (terminals per CTA / records per staged tile of
-the exhaustive scans), HAC_CM_WARPS (warps per block of the cache update).
+the exhaustive scans), HAC_CM_WARPS (warps per block of the cache update),
+HAC_GS_W2 / HAC_GS_W / HAC_GS_N / HAC_GS_WIDE (group sizes of the grouped search
+in d <= 2, above, and below HAC_GS_WIDE terminals), HAC_GS_CUT / HAC_GS_GW (binary
+orders of radius past which a terminal is searched alone / warps per block).
 """
 from __future__ import annotations
 
@@ -43,7 +46,8 @@ import statistics
 
 
 SHAPES = ("HAC_DS_PPT8", "HAC_DS_MINB", "HAC_QWARPS", "HAC_QMINB", "HAC_QMINB_COMPLETE", "HAC_Q_OUTLINE", "HAC_BR_T",
-          "HAC_BR_C", "HAC_CM_WARPS")
+          "HAC_BR_C", "HAC_CM_WARPS", "HAC_GS_W", "HAC_GS_W2", "HAC_GS_N", "HAC_GS_WIDE", "HAC_GS_CUT",
+          "HAC_GS_GW")
 
 
 def shape_grid(spec: str):
