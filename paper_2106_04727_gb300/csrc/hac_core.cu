@@ -1465,7 +1465,7 @@ int init_layout(hac_ctx *h, cudaStream_t st) {
     double lo = dec(bb[k]), hi = dec(bb[MAXD + k]);
     mp.lo[k] = lo;
     mp.inv[k] = hi > lo ? 1.0 / (hi - lo) : 0.0;
-    ctrp.lo[k] = 0.5 * (lo + hi);
+    ctrp.lo[k] = box_centre(lo, hi);
     scale = std::max(scale, std::max(std::fabs(lo - ctrp.lo[k]), std::fabs(hi - ctrp.lo[k])));
     raw = std::max(raw, std::max(std::fabs(lo), std::fabs(hi)));
   }

@@ -309,7 +309,7 @@ __device__ bool fin_start(const FinArgs &a, const FinSm &m, double *s_box, float
   }
   double scale = 0.0;
   for (int k = 0; k < d; ++k) {
-    const double c = 0.5 * (s_box[k] + s_box[MAXD + k]);
+    const double c = box_centre(s_box[k], s_box[MAXD + k]);
     scale = fmax(scale, fmax(fabs(s_box[k] - c), fabs(s_box[MAXD + k] - c)));
   }
   const int ue = unit_exp(scale);
@@ -327,12 +327,12 @@ __device__ bool fin_start(const FinArgs &a, const FinSm &m, double *s_box, float
 #pragma unroll
     for (int k = 0; k < D; ++k)
       m.x[k * a.Kc + i] =
-          k < d ? (float)(((double)X[(size_t)i * d + k] - 0.5 * (s_box[k] + s_box[MAXD + k])) * mul)
+          k < d ? (float)(((double)X[(size_t)i * d + k] - box_centre(s_box[k], s_box[MAXD + k])) * mul)
                 : 0.f;
   }
   for (int i = cta_rank() * FT + threadIdx.x; i < n; i += cta_count() * FT) {
     for (int k = 0; k < d; ++k) {
-      const double x = ((double)X[(size_t)i * d + k] - 0.5 * (s_box[k] + s_box[MAXD + k])) * mul;
+      const double x = ((double)X[(size_t)i * d + k] - box_centre(s_box[k], s_box[MAXD + k])) * mul;
       s.csum[(size_t)i * dp + k] = x;
       s.cent[(size_t)i * dp + k] = x;
       s.cent32[(size_t)i * dp + k] = (float)x;

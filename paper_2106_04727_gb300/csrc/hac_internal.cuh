@@ -343,6 +343,8 @@ __host__ __device__ inline int unit_exp(double scale) {
   frexp(scale, &e);
   return e < -1023 ? -1023 : e > 1023 ? 1023 : e;
 }
+// the middle of [lo, hi] (halved first: the sum may be beyond FP64)
+__host__ __device__ inline double box_centre(double lo, double hi) { return 0.5 * lo + 0.5 * hi; }
 // a height in input units (avg-2: squared units)
 __host__ __device__ inline double unit_height(double h, double unit, bool squared) {
   h *= unit;

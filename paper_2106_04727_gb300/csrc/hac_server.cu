@@ -405,7 +405,7 @@ int engine_admit(Engine &e, const std::vector<SrvReq *> &batch) {
     for (int k = 0; k < MAXD; ++k) {
       a.lo[k] = k < d ? lo[k] : 0.0;
       a.inv[k] = k < d && hi[k] > lo[k] ? 1.0 / (hi[k] - lo[k]) : 0.0;
-      a.ctr[k] = k < d ? 0.5 * (lo[k] + hi[k]) : 0.0;
+      a.ctr[k] = k < d ? box_centre(lo[k], hi[k]) : 0.0;
       if (k < d)
         scale = std::max(scale, std::max(std::fabs(lo[k] - a.ctr[k]), std::fabs(hi[k] - a.ctr[k])));
     }

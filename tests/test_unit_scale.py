@@ -86,3 +86,23 @@ def test_fp32_mode(lk, entry, k, dt, monkeypatch):
         got["h"] = np.ldexp(got["h"], -2 * k if lk == "average_sq" else -k)
     c = oracle.compare(got, oracle.nnchain(X.astype(np.float64), lk), rtol=1e-5)
     assert c["ok"], c
+
+
+@pytest.mark.parametrize("entry", list(CALLS))
+@pytest.mark.parametrize("lk", LKS)
+def test_next_to_the_largest_number(lk, entry, monkeypatch):
+    """All coordinates near 1.5 * 10^308: the sum of the box's ends is beyond FP64."""
+    if entry == "tree":
+        monkeypatch.setenv("HAC_DENSE_K", "0")
+    Y = inputs.gaussian_mixture(300, 2, 4, seed=19, dtype=np.float64)
+    X = np.ldexp(Y, 1010) + 1.5e308
+    Y = np.ldexp(X, -1010) - np.ldexp(1.5e308, -1010)   # the same points, exactly
+    got = CALLS[entry](X, lk, hac.PREC_F64)
+    want = oracle.nnchain(Y, lk)
+    if lk == "average_sq":   # heights are beyond FP64: the merges by size and order
+        assert np.all(np.isinf(got["h"][want["h"] > 1e-3]))
+        assert sorted(zip(got["a"], got["b"])) == sorted(zip(want["a"], want["b"]))
+        return
+    got["h"] = np.ldexp(got["h"], -1010)
+    c = oracle.compare(got, want, rtol=1e-9)
+    assert c["ok"], c
