@@ -179,9 +179,11 @@ __device__ __forceinline__ U128 u128_shfl_xor(const U128 &v, int o) {
 // A finished sum is two words (lo, hi), the estimate flag in the top bit of hi.
 // The mean distance of an entry, one function everywhere so that equal sums
 // and sizes give equal means, whichever cluster has which size: the 128-bit
-// sum as the nearest FP64 number (to even), times the product of 1 / size of
-// both (reciprocals kept per matrix index: no FP64 division); the sign bit
-// set for an estimate.  The FP64 pipe (2 lanes per clock and SM)
+// sum as the nearest FP64 number (to even), times 1 / size of the smaller
+// cluster, times 1 / size of the other (reciprocals kept per matrix index: no
+// FP64 division; one at a time, not their product, so that a sum that the sizes
+// divide gives the whole quotient and true ties of lattice points stay ties);
+// the sign bit set for an estimate.  The FP64 pipe (2 lanes per clock and SM)
 // bounds every kernel that makes means, so the sum is converted by integer
 // instructions and two FP64 multiplications are left: the matrix rebuild at
 // 16,106 clusters took 1.90 ms with the seven FP64 instructions of two integer
@@ -215,7 +217,10 @@ __device__ __forceinline__ double sum_double(unsigned long long hi, unsigned lon
 }
 
 __device__ __forceinline__ double entry_mean(const U128 &v, int e, double inv_a, double inv_b) {
-  const double m = sum_double(v.hi & ~TOP, v.lo, e) * (inv_a * inv_b);
+  // (ordered by integer comparisons: bits of positive numbers)
+  const long long a = __double_as_longlong(inv_a), c = __double_as_longlong(inv_b);
+  const double m = sum_double(v.hi & ~TOP, v.lo, e) * __longlong_as_double(max(a, c)) *
+                   __longlong_as_double(min(a, c));
   const unsigned long long b = (unsigned long long)__double_as_longlong(m);
   return __longlong_as_double((long long)(v.hi & TOP ? (b | SIGN) : b));
 }
