@@ -7,6 +7,7 @@
 #include "hac_dev.cuh"
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -19,6 +20,27 @@ namespace hacg {
 constexpr int TPB = 256;
 
 __host__ __device__ inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
+
+// Bounds, summaries and screening square coordinates in FP32, so the clustering
+// runs at a scale that FP32 holds: an input whose largest recentred coordinate is
+// outside [FIN_SCALE_LO, FIN_SCALE_HI) is multiplied by 2^-unit_exp, which takes
+// it to [0.5, 1), and heights are multiplied back as they leave (both exact,
+// unless a height itself is outside FP64's normal range).  Unscaled, coordinates
+// from 2^63 on had infinite lower bounds and lost their nearest neighbours, and
+// below 2^-50 every FP32 variance was the least subnormal.
+__host__ __device__ inline int unit_exp(double scale) {
+  if (!(scale > 0.0) || (scale >= FIN_SCALE_LO && scale < FIN_SCALE_HI)) return 0;
+  int e;
+  frexp(scale, &e);
+  return e < -1023 ? -1023 : e > 1023 ? 1023 : e;
+}
+// the middle of [lo, hi] (halved first: the sum may be beyond FP64)
+__host__ __device__ inline double box_centre(double lo, double hi) { return 0.5 * lo + 0.5 * hi; }
+// a height in input units (avg-2: squared units)
+__host__ __device__ inline double unit_height(double h, double unit, bool squared) {
+  h *= unit;
+  return squared ? h * unit : h;
+}
 
 // ---------------------------------------------------------------------------
 // pair-distance cache slots (Section 5): the write protocol

@@ -7,7 +7,6 @@
 #pragma once
 
 #include <cuda_runtime.h>
-#include <math.h>
 #include <stdint.h>
 
 namespace hacg {
@@ -139,7 +138,7 @@ struct State {
   float *islack;        // absolute pruning slack (coordinate scale * 2^-18)
   float *iscale;        // largest |coordinate| after recentring
   float *idpts;         // error term of FP32 point distances (0 for FP32 input)
-  double *iunit;        // input units per unit of the clustered coordinates (unit_exp)
+  double *iunit;        // input units per unit of the clustered coordinates (unit_exp, hac_impl.cuh)
   int32_t *irec;        // first merge-record slot (= first cid of the instance)
   int32_t *irecn;       // merge records written
   int32_t *iact;        // active clusters left
@@ -329,27 +328,6 @@ constexpr int FIN_MAX_K = 4096;
 constexpr int FIN_SMEM = 200 * 1024;
 constexpr double FIN_SCALE_LO = 9.313225746154785e-10;  // 2^-30
 constexpr double FIN_SCALE_HI = 1099511627776.0;        // 2^40
-
-// Bounds, summaries and screening square coordinates in FP32, so the clustering
-// runs at a scale that FP32 holds: an input whose largest recentred coordinate is
-// outside [FIN_SCALE_LO, FIN_SCALE_HI) is multiplied by 2^-unit_exp, which takes
-// it to [0.5, 1), and heights are multiplied back as they leave (both exact,
-// unless a height itself is outside FP64's normal range).  Unscaled, coordinates
-// from 2^63 on had infinite lower bounds and lost their nearest neighbours, and
-// below 2^-50 every FP32 variance was the least subnormal.
-__host__ __device__ inline int unit_exp(double scale) {
-  if (!(scale > 0.0) || (scale >= FIN_SCALE_LO && scale < FIN_SCALE_HI)) return 0;
-  int e;
-  frexp(scale, &e);
-  return e < -1023 ? -1023 : e > 1023 ? 1023 : e;
-}
-// the middle of [lo, hi] (halved first: the sum may be beyond FP64)
-__host__ __device__ inline double box_centre(double lo, double hi) { return 0.5 * lo + 0.5 * hi; }
-// a height in input units (avg-2: squared units)
-__host__ __device__ inline double unit_height(double h, double unit, bool squared) {
-  h *= unit;
-  return squared ? h * unit : h;
-}
 
 // dimension a record is staged with (zero-padded to it), and its bytes: the
 // coordinates, 1/size or variance, cid and terminal entry
