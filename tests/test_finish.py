@@ -1,7 +1,7 @@
 """The one-launch rounds of Ward and avg-2 (csrc/hac_finish.cu): whole runs from
 the points, and the last rounds of larger runs, against the CPU oracle merge
 for merge and round for round; block counts, the capacity and what lies just
-beyond it; ties; scales the FP32 screening does not take; round limits."""
+beyond it; ties; scales the FP32 screening would not hold; round limits."""
 import numpy as np
 import pytest
 
@@ -50,8 +50,8 @@ def test_ties_and_duplicates(lk):
 @pytest.mark.parametrize("lk", LKS)
 @pytest.mark.parametrize("scale", [1e-11, 1e-8, 1e11, 1e14])
 def test_scales(lk, scale):
-    """Far from 1 the FP32 squares would flush or overflow: those inputs take
-    the ordinary rounds; next to the limits the screening still holds."""
+    """Far from 1 the FP32 squares would flush or overflow: those inputs are
+    clustered at another scale; next to the limits the screening still holds."""
     X = inputs.gaussian_mixture(300, 3, 4, seed=8, dtype=np.float64) * (scale / 50.0)
     _check(hac.cluster(X, lk), oracle.rounds(X, lk))
 
