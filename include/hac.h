@@ -172,7 +172,8 @@ int hac_create_device(const void *dev_points, int64_t n, int d, hac_dtype dt, ha
  * Section 5 cache with room for every pair: 24 bytes per entry of the K x K
  * matrix, allocated once per handle; without room for it the run stays on
  * the range-query search).  K is 4,096 to 8,192 for d <= 3 and 4,096 to 16,384
- * for d <= 8, by n, and 65,536 above, capped so that the matrix takes at most
+ * for d <= 8, by n, and 20,000 to 65,536 above (32,768 for up to that many
+ * points), capped so that the matrix takes at most
  * half of the device memory free when the run starts.  Complete linkage runs
  * on such a matrix (16 bytes per entry) from the first round on if it has at
  * most K points: 24,576 to 32,768 by d and precision, capped the same way.  A
